@@ -38,11 +38,11 @@ struct WsHeader {
 };
 static_assert(sizeof(WsHeader) == 256, "header is one 256-byte segment");
 
-// Partial sums of one block of the statistics reduction.
+// Partial results of one block of the statistics reduction: nine sums, five
+// counts (exact integers), minimum and maximum ratio.
+constexpr int kStatFields = 16;
 struct StatPart {
-  double s_ell, s_pg, s_k3, s_H, s_r, s_rabs, s_lpabs, s_rc, s_rcabs;
-  float rmin, rmax;
-  unsigned long long n, n_hi, n_lo, n_dual, n_corr;
+  double f[kStatFields];
 };
 
 constexpr int kMaxTopK = 64;
@@ -273,6 +273,22 @@ __device__ __forceinline__ uint32_t cluster_nctarank() {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Programmatic dependent launch. A kernel launched as a programmatic
+// dependent of the one before it in the stream may start once every CTA of
+// that kernel has called pdl_trigger (or has exited); pdl_wait then waits
+// until that kernel has finished and its writes are visible. The first kernel
+// of every call is launched as an ordinary kernel, so nothing of an earlier
+// call, or of the caller's, is still running when a call's kernels start, and
+// every kernel launched as a dependent calls pdl_wait before it reads or
+// writes anything that an earlier kernel of the call touches: inputs of the
+// call may be read before it. (Without the launch attribute both are no-ops.)
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {

@@ -4,13 +4,19 @@
 // training tokens of every trajectory, and validation of group ids and row
 // offsets.
 //
-// One CTA of 1024 threads does all of it: the inputs are a few KB of
-// per-trajectory data plus one byte and one float per row. Row offsets,
-// per-trajectory counts and advantages are staged in shared memory when they
-// fit. The row passes go one warp per trajectory over its contiguous rows.
+// The inputs are a few KB of per-trajectory data plus one byte and one float
+// per row, so what bounds the kernel is latency: the chain of loads, the
+// double-precision group statistics (GB300 runs double precision at about two
+// operations per SM and clock) and, past some ten thousand rows, one SM's
+// loads and stores. One thread-block cluster of up to kAdvCluster CTAs does
+// all of it: groups and trajectories are spread over its warps, counts are
+// added with integer atomics, and two cluster barriers separate the group
+// statistics, the row passes and (REINFORCE++) the normalisation. The sweep
+// that follows is launched as a programmatic dependent (pdl_trigger below), so
+// its first pass over the logits runs meanwhile.
 // Every floating-point sum runs in a fixed order (lane-strided partial sums,
 // xor-butterfly merges) in double precision and every count is an integer, so
-// results are bit-for-bit reproducible.
+// results are bit-for-bit reproducible, whatever the cluster's size.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -25,92 +31,76 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ int warp_sum_i(int v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-__device__ __forceinline__ double warp_min(double v) {
+__device__ __forceinline__ float warp_maxf(float v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
 
-// Block-wide sums in a fixed order (valid in every thread).
-__device__ double block_sum(double v, double* sh) {
+// Block-wide sum / maximum in a fixed order (valid in every thread): warp
+// butterflies, then every warp merges the warps' values by another (one
+// double operation per step and warp; a serial loop over the warps in every
+// thread queued 32 x 32 of them on the SM's double unit, 8 us a sum).
+template <bool kMax>
+__device__ double block_merge_d(double v, double* sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  v = warp_sum(v);
+  v = kMax ? warp_max(v) : warp_sum(v);
   __syncthreads();
   if (lane == 0) sh[warp] = v;
   __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < kWarps; ++w) t += sh[w];
-  return t;
-}
-// Exact integer block sum (valid in every thread).
-__device__ unsigned long long block_sum_u(unsigned long long v, unsigned long long* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) sh[warp] = v;
-  __syncthreads();
-  unsigned long long t = 0;
-  for (int w = 0; w < kWarps; ++w) t += sh[w];
-  return t;
-}
-__device__ double block_max(double v, double* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  v = warp_max(v);
-  __syncthreads();
-  if (lane == 0) sh[warp] = v;
-  __syncthreads();
-  double t = -INFINITY;
-  for (int w = 0; w < kWarps; ++w) t = fmax(t, sh[w]);
-  return t;
+  double t = lane < kWarps ? sh[lane] : (kMax ? -INFINITY : 0.0);
+  return kMax ? warp_max(t) : warp_sum(t);
 }
 
 // The statistics of group g, computed by one warp that scans the group ids
 // for the group's members: n, mean, the standard deviation with its floor,
-// and whether all rewards are equal. In double precision.
+// and whether all rewards are equal. In double precision; a step of the scan
+// that meets no member adds nothing and skips the double arithmetic.
 __device__ void group_stats(const AdvArgs& a, const int* gid, const float* rew, int g, int lane) {
   WsPtrs ws = a.ws;
   int n = 0;
-  double sum = 0.0, wmax = -INFINITY, wmin = INFINITY;
+  double sum = 0.0;
+  float wmax = -INFINITY, wmin = INFINITY;
 #pragma unroll 4
-  for (int i = lane; i < a.n_traj; i += 32) {
-    if (gid[i] == g) {
-      const double w = rew[i];
+  for (int b = 0; b < a.n_traj; b += 32) {
+    const int i = b + lane;
+    const bool in = i < a.n_traj && gid[i] == g;
+    if (!__any_sync(0xffffffffu, in)) continue;
+    if (in) {
+      const float w = rew[i];
       ++n;
-      sum += w;
-      wmax = fmax(wmax, w);
-      wmin = fmin(wmin, w);
+      sum += static_cast<double>(w);
+      wmax = fmaxf(wmax, w);
+      wmin = fminf(wmin, w);
     }
   }
-  n = warp_sum_i(n);
+  n = __reduce_add_sync(0xffffffffu, n);
   sum = warp_sum(sum);
-  wmax = warp_max(wmax);
-  wmin = warp_min(wmin);
+  wmax = warp_maxf(wmax);
+  wmin = -warp_maxf(-wmin);
   const double mu = n > 0 ? sum / n : 0.0;
-  double ss = 0.0;
-#pragma unroll 4
-  for (int i = lane; i < a.n_traj; i += 32) {
-    if (gid[i] == g) {
-      const double d = static_cast<double>(rew[i]) - mu;
-      ss += d * d;
-    }
-  }
-  ss = warp_sum(ss);
   // A group whose rewards are all equal (this includes one-member groups)
   // carries no advantage signal: its GRPO advantages are exactly zero.
   const int flat = (n == 0) || (wmax == wmin);
   double den = 1.0;
-  if (a.normalize_std && !flat) {
+  if (a.normalize_std && !flat) {  // (uniform over the warp)
+    double ss = 0.0;
+#pragma unroll 4
+    for (int b = 0; b < a.n_traj; b += 32) {
+      const int i = b + lane;
+      const bool in = i < a.n_traj && gid[i] == g;
+      if (!__any_sync(0xffffffffu, in)) continue;
+      if (in) {
+        const double d = static_cast<double>(rew[i]) - mu;
+        ss += d * d;
+      }
+    }
+    ss = warp_sum(ss);
     const int ddof = a.unbiased_std ? 1 : 0;
     den = fmax(sqrt(ss / static_cast<double>(n - ddof)), static_cast<double>(a.std_floor));
   }
@@ -122,10 +112,8 @@ __device__ void group_stats(const AdvArgs& a, const int* gid, const float* rew, 
   }
 }
 
-// Group statistics for calls with more than kInlineGroups groups, one
-// 32-thread block per group. GB300 runs double precision at a small fraction
-// of its fp32 rate: spread over the SMs, the groups' double arithmetic no
-// longer queues on the one SM that runs k_advantages.
+// Group statistics for calls whose groups are too many for one cluster
+// (group_kernel_pays), one 32-thread block per group over the whole GPU.
 __global__ void __launch_bounds__(32) k_groups(const AdvArgs a) {
   for (int g = blockIdx.x; g < a.n_groups; g += gridDim.x)
     group_stats(a, a.gid, a.rewards, g, threadIdx.x);
@@ -133,57 +121,67 @@ __global__ void __launch_bounds__(32) k_groups(const AdvArgs a) {
 
 __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) {
   extern __shared__ __align__(16) int dyn[];
+  pdl_trigger();  // (launched as an ordinary kernel: whatever ran before it has finished)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = static_cast<int>(cluster_ctarank()), NC = static_cast<int>(cluster_nctarank());
+  const int gtid = rank * kAdvThreads + tid, gthreads = NC * kAdvThreads;
+  const int gwarp = rank * kWarps + warp, gwarps = NC * kWarps;
   __shared__ unsigned int s_err;
   __shared__ double s_red[kWarps];
-  __shared__ unsigned long long s_cnt[kWarps];
+  __shared__ unsigned long long s_tok;
+  __shared__ unsigned int s_seq;
   WsPtrs ws = a.ws;
-  // Shared copies, when they fit, of cu (n_traj + 1), the per-trajectory
-  // token counts and advantages, group ids and rewards (n_traj each).
+  // Shared copies, when they fit, of cu (n_traj + 1), group ids and rewards.
   const bool on_chip = a.smem_traj;
   const int nt = a.n_traj;
-  int* cu = on_chip ? dyn : const_cast<int*>(a.cu);
-  int* cnt_i = on_chip ? dyn + (nt + 1) : ws.traj_n;
-  const int* gid = on_chip ? dyn + (3 * nt + 1) : a.gid;
-  const float* rew = on_chip ? reinterpret_cast<const float*>(dyn + (4 * nt + 1)) : a.rewards;
+  const int* cu = on_chip ? dyn : a.cu;
+  const int* gid = on_chip ? dyn + (nt + 1) : a.gid;
+  const float* rew = on_chip ? reinterpret_cast<const float*>(dyn + (2 * nt + 1)) : a.rewards;
   if (tid == 0) {
     s_err = 0;
-    ws.hdr->err_bits = 0;
-    ws.hdr->ticket = 0;
+    s_tok = 0;
+    s_seq = 0;
+    if (rank == 0) {
+      ws.hdr->err_bits = 0;
+      ws.hdr->ticket = 0;
+      ws.hdr->n_tokens = 0;
+      ws.hdr->n_seq = 0;
+    }
   }
-  for (int i = tid; i <= nt; i += kAdvThreads) {
-    if (on_chip) {
-      cu[i] = a.cu[i];
+  if (on_chip)
+    for (int i = tid; i <= nt; i += kAdvThreads) {
+      dyn[i] = a.cu[i];
       if (i < nt) {
-        dyn[3 * nt + 1 + i] = a.gid[i];
-        reinterpret_cast<float*>(dyn + 4 * nt + 1)[i] = a.rewards[i];
+        dyn[nt + 1 + i] = a.gid[i];
+        reinterpret_cast<float*>(dyn + 2 * nt + 1)[i] = a.rewards[i];
       }
     }
-    if (i < nt) cnt_i[i] = 0;
+  for (int i = gtid; i < nt; i += gthreads) {
+    ws.traj_n[i] = 0;
+    if (a.counts_out) a.counts_out[i] = 0;
   }
   __syncthreads();
 
-  // ---- validation
+  // ---- validation (every CTA reads all of the row offsets)
   unsigned int err = 0;
-  for (int i = tid; i < a.n_traj; i += kAdvThreads) {
+  for (int i = tid; i < nt; i += kAdvThreads) {
     if (cu[i] > cu[i + 1]) err |= kErrSeqlens;
     const int g = gid[i];
     if (g < 0 || g >= a.n_groups) err |= kErrGroup;
   }
-  if (tid == 0 && (cu[0] != 0 || static_cast<long long>(cu[a.n_traj]) != a.R_total))
-    err |= kErrSeqlens;
+  if (tid == 0 && (cu[0] != 0 || static_cast<long long>(cu[nt]) != a.R_total)) err |= kErrSeqlens;
   if (err) atomicOr(&s_err, err);
 
-  // ---- group statistics: one warp per group here when there are few
-  // (otherwise k_groups computed them just before)
-  if (a.n_groups <= kInlineGroups)
-    for (int g = warp; g < a.n_groups; g += kWarps) group_stats(a, gid, rew, g, lane);
+  // ---- group statistics, one warp per group
+  if (!a.groups_done)
+    for (int g = gwarp; g < a.n_groups; g += gwarps) group_stats(a, gid, rew, g, lane);
+  // every CTA's part of the header, the counts and the group table is written
   __syncthreads();
+  cluster_sync_all();
   const bool cu_ok = (s_err & kErrSeqlens) == 0;
   const bool rpp = a.estimator == RL_EST_REINFORCEPP || a.estimator == RL_EST_REINFORCEPP_BASELINE;
 
-  // ---- per-trajectory base value (kept in double in a register-free way:
-  // recomputed from the group table where needed)
+  // ---- a trajectory's base value, in double from the group table
   auto base_value = [&](int i) -> double {
     const int g = gid[i];
     const bool gok = g >= 0 && g < a.n_groups;
@@ -193,32 +191,23 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
     if (!gok || ws.g_flag[g]) return 0.0;  // GRPO, GSPO
     return (w - ws.g_mu[g]) / ws.g_den[g];
   };
-
-  // Trajectory advantages (in shared memory when the trajectory tables fit).
-  float* a_s = on_chip ? reinterpret_cast<float*>(dyn + 2 * a.n_traj + 1) : ws.a_traj;
-  auto publish = [&](int i, double A) {
-    a_s[i] = static_cast<float>(A);
-    if (on_chip) ws.a_traj[i] = static_cast<float>(A);
-    if (a.advantages) a.advantages[i] = static_cast<float>(A);
+  auto publish = [&](int i, float A) {
+    ws.a_traj[i] = A;
+    if (a.advantages) a.advantages[i] = A;
   };
-  // GRPO and GSPO: the trajectory advantage is final before any row is read,
-  // so one pass over the rows counts and writes the row advantages.
-  if (!rpp) {
-    for (int i = tid; i < a.n_traj; i += kAdvThreads) publish(i, base_value(i));
-    __syncthreads();
-  }
 
   // ---- passes over the rows, one warp per trajectory (its rows are the
   // contiguous range [cu[i], cu[i+1]); several warps per trajectory when
   // there are fewer trajectories than warps): the lanes count the trajectory's
   // training tokens from 16-byte blocks of the mask and fill its row
-  // advantages with 16-byte stores, with the one-sample OPD shaping. With
-  // invalid row offsets every row gets advantage 0 (plus the shaping) and
-  // only N is counted, row by row. A shard sees the part of each trajectory
-  // that falls in its rows [row0, row0 + R) (local indices from 0); given the
-  // counts of every shard (counts_in), it takes N and the trajectories'
-  // counts from them instead of counting.
-  const bool lookup = cu_ok && a.n_traj > 0;
+  // advantages with 16-byte stores, with the one-sample OPD shaping. GRPO and
+  // GSPO know the advantage here and make both in one pass. With invalid row
+  // offsets every row gets advantage 0 (plus the shaping) and only N is
+  // counted, row by row. A shard sees the part of each trajectory that falls
+  // in its rows [row0, row0 + R) (local indices from 0); given the counts of
+  // every shard (counts_in), it takes N and the trajectories' counts from
+  // them instead of counting.
+  const bool lookup = cu_ok && nt > 0;
   const bool mask_vec = (reinterpret_cast<uintptr_t>(a.mask) & 15u) == 0;
   const bool row_vec = (reinterpret_cast<uintptr_t>(ws.a_row) & 15u) == 0;
   const bool opd_vec = a.teacher && ((reinterpret_cast<uintptr_t>(a.rho) |
@@ -231,11 +220,12 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
   };
   // With fewer trajectories than warps, wpt warps share each trajectory
   // (warp `sub` of them takes every wpt-th 512-row or 128-row piece).
-  const int wpt = a.n_traj > 0 ? max(1, kWarps / a.n_traj) : 1;
-  const int traj_groups = kWarps / wpt;
-  const int group = warp / wpt, sub = warp % wpt;
+  const int wpt = nt > 0 ? max(1, gwarps / nt) : 1;
+  const int traj_groups = gwarps / wpt;
+  const int group = gwarp / wpt, sub = gwarp % wpt;
   auto count_rows = [&](long long lo, long long hi) {  // training tokens in [lo, hi), warp-wide
     int c = 0;
+#pragma unroll 2
     for (long long b = (lo & ~15LL) + 16LL * (lane + 32 * sub); b < hi; b += 16LL * 32 * wpt) {
       if (mask_vec && b >= lo && b + 16 <= hi) {
         const uint4 v = *reinterpret_cast<const uint4*>(a.mask + b);
@@ -245,9 +235,10 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
         for (long long t = max(b, lo); t < min(b + 16, hi); ++t) c += a.mask[t] != 0;
       }
     }
-    return warp_sum_i(c);
+    return static_cast<int>(__reduce_add_sync(0xffffffffu, c));
   };
   auto write_rows = [&](long long lo, long long hi, float A) {  // row advantages of [lo, hi)
+#pragma unroll 2
     for (long long b = (lo & ~3LL) + 4LL * (lane + 32 * sub); b < hi; b += 4LL * 32 * wpt) {
       if (row_vec && b >= lo && b + 4 <= hi && (!a.teacher || opd_vec)) {
         float4 v = make_float4(A, A, A, A);
@@ -265,94 +256,97 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
       }
     }
   };
-  unsigned long long n_tok = 0;
-  if (lookup && a.counts_in) {
-    for (int i = tid; i < a.n_traj; i += kAdvThreads) {
-      const int c = a.counts_in[i];
-      cnt_i[i] = c;
-      n_tok += static_cast<unsigned long long>(c);
-    }
-    if (!rpp && group < traj_groups)
-      for (int i = group; i < a.n_traj; i += traj_groups) write_rows(local_lo(i), local_hi(i), a_s[i]);
-    __syncthreads();
-  } else if (lookup) {
-    if (group < traj_groups) {
-      for (int i = group; i < a.n_traj; i += traj_groups) {
-        const long long lo = local_lo(i), hi = local_hi(i);
-        const int c = count_rows(lo, hi);
-        if (lane == 0 && c) {
-          atomicAdd(&cnt_i[i], c);  // integer: exact in any order
-          n_tok += static_cast<unsigned long long>(c);
-        }
-        if (!rpp) write_rows(lo, hi, a_s[i]);
+  unsigned long long n_tok = 0;  // (lane 0 of each warp, or every thread's own)
+  unsigned int n_seq = 0;
+  if (lookup) {
+    if (a.counts_in)
+      for (int i = gtid; i < nt; i += gthreads) {
+        const int c = a.counts_in[i];
+        ws.traj_n[i] = c;
+        n_tok += static_cast<unsigned long long>(c);
+        n_seq += c > 0;
       }
-    }
-    __syncthreads();  // every trajectory's count complete
-    if (a.counts_out)
-      for (int i = tid; i < a.n_traj; i += kAdvThreads) a.counts_out[i] = cnt_i[i];
+    if (group < traj_groups)
+      for (int i = group; i < nt; i += traj_groups) {
+        const long long lo = local_lo(i), hi = local_hi(i);
+        if (!a.counts_in) {
+          const int c = count_rows(lo, hi);
+          if (lane == 0 && c) {  // integers: exact in any order
+            n_seq += atomicAdd(&ws.traj_n[i], c) == 0;
+            if (a.counts_out) atomicAdd(&a.counts_out[i], c);
+            n_tok += static_cast<unsigned long long>(c);
+          }
+        }
+        if (!rpp) {
+          const float A = static_cast<float>(base_value(i));
+          if (sub == 0 && lane == 0) publish(i, A);
+          write_rows(lo, hi, A);
+        }
+      }
   } else {
-    for (long long t = tid; t < a.R; t += kAdvThreads) {
+    for (long long t = gtid; t < a.R; t += gthreads) {
       n_tok += a.mask[t] != 0;
       if (!rpp) ws.a_row[t] = -opd(t);
     }
+    for (int i = gtid; i < nt; i += gthreads)
+      if (!rpp) publish(i, static_cast<float>(base_value(i)));
   }
-  const double N = static_cast<double>(block_sum_u(n_tok, s_cnt));
-
-  // ---- REINFORCE++: normalise the returns over the training tokens, then
-  // a second pass writes the row advantages
-  if (rpp) {
-    double sb = 0.0, bmax = -INFINITY, bmin = INFINITY;
-    for (int i = tid; i < a.n_traj; i += kAdvThreads) {
-      const int n_i = cnt_i[i];
-      if (n_i == 0) continue;
-      const double b = base_value(i);
-      sb += b * n_i;
-      bmax = fmax(bmax, b);
-      bmin = fmin(bmin, b);
-    }
-    sb = block_sum(sb, s_red);
-    bmax = block_max(bmax, s_red);
-    bmin = -block_max(-bmin, s_red);
-    const bool zero_all = !(N > 0.0) || !(bmax != bmin);
-    const double mu = N > 0.0 ? sb / N : 0.0;
-    double ss = 0.0;
-    for (int i = tid; i < a.n_traj; i += kAdvThreads) {
-      const int n_i = cnt_i[i];
-      if (n_i == 0) continue;
-      const double d = base_value(i) - mu;
-      ss += d * d * n_i;
-    }
-    ss = block_sum(ss, s_red);
-    double den = 1.0;
-    if (a.normalize_std) {
-      const double ddof = a.unbiased_std ? 1.0 : 0.0;
-      const double var = N > ddof ? ss / (N - ddof) : 0.0;
-      den = fmax(sqrt(var), static_cast<double>(a.std_floor));
-    }
-    for (int i = tid; i < a.n_traj; i += kAdvThreads)
-      publish(i, zero_all ? 0.0 : (base_value(i) - mu) / den);
-    __syncthreads();
-    if (lookup) {
-      if (group < traj_groups)
-        for (int i = group; i < a.n_traj; i += traj_groups)
-          write_rows(local_lo(i), local_hi(i), a_s[i]);
-    } else {
-      for (long long t = tid; t < a.R; t += kAdvThreads) ws.a_row[t] = -opd(t);
-    }
-  }
-
-  // ---- the training tokens of each trajectory, and how many trajectories train
-  int n_seq = 0;
-  for (int i = tid; i < a.n_traj; i += kAdvThreads) {
-    const int n_i = cnt_i[i];
-    if (on_chip) ws.traj_n[i] = n_i;
-    n_seq += (n_i > 0);
-  }
-  const unsigned long long n_seq_all = block_sum_u(static_cast<unsigned long long>(n_seq), s_cnt);
+  if (n_tok) atomicAdd(&s_tok, n_tok);
+  if (n_seq) atomicAdd(&s_seq, n_seq);
+  __syncthreads();
   if (tid == 0) {
-    ws.hdr->n_tokens = static_cast<long long>(N);
-    ws.hdr->n_seq = static_cast<long long>(n_seq_all);  // exact integer counts
+    if (s_tok) atomicAdd(reinterpret_cast<unsigned long long*>(&ws.hdr->n_tokens), s_tok);
+    if (s_seq)
+      atomicAdd(reinterpret_cast<unsigned long long*>(&ws.hdr->n_seq),
+                static_cast<unsigned long long>(s_seq));
     if (s_err) atomicOr(&ws.hdr->err_bits, s_err);
+  }
+  if (!rpp) return;
+
+  // ---- REINFORCE++: normalise the returns over the training tokens, then a
+  // second pass writes the row advantages. Every CTA forms the moments, over
+  // all trajectories in the same order.
+  __syncthreads();
+  cluster_sync_all();  // every CTA's counts are in
+  const double N = static_cast<double>(__ldcg(&ws.hdr->n_tokens));
+  double sb = 0.0, bmax = -INFINITY, bmin = INFINITY;
+  for (int i = tid; i < nt; i += kAdvThreads) {
+    const int n_i = __ldcg(&ws.traj_n[i]);
+    if (n_i == 0) continue;
+    const double b = base_value(i);
+    sb += b * n_i;
+    bmax = fmax(bmax, b);
+    bmin = fmin(bmin, b);
+  }
+  sb = block_merge_d<false>(sb, s_red);
+  bmax = block_merge_d<true>(bmax, s_red);
+  bmin = -block_merge_d<true>(-bmin, s_red);
+  const bool zero_all = !(N > 0.0) || !(bmax != bmin);
+  const double mu = N > 0.0 ? sb / N : 0.0;
+  double ss = 0.0;
+  for (int i = tid; i < nt; i += kAdvThreads) {
+    const int n_i = __ldcg(&ws.traj_n[i]);
+    if (n_i == 0) continue;
+    const double d = base_value(i) - mu;
+    ss += d * d * n_i;
+  }
+  ss = block_merge_d<false>(ss, s_red);
+  double den = 1.0;
+  if (a.normalize_std) {
+    const double ddof = a.unbiased_std ? 1.0 : 0.0;
+    const double var = N > ddof ? ss / (N - ddof) : 0.0;
+    den = fmax(sqrt(var), static_cast<double>(a.std_floor));
+  }
+  auto final_value = [&](int i) {
+    return static_cast<float>(zero_all ? 0.0 : (base_value(i) - mu) / den);
+  };
+  for (int i = gtid; i < nt; i += gthreads) publish(i, final_value(i));
+  if (lookup) {
+    if (group < traj_groups)
+      for (int i = group; i < nt; i += traj_groups)
+        write_rows(local_lo(i), local_hi(i), final_value(i));
+  } else {
+    for (long long t = gtid; t < a.R; t += gthreads) ws.a_row[t] = -opd(t);
   }
 }
 

@@ -17,11 +17,8 @@ template <class In, class Out>
 __global__ void __launch_bounds__(kBwdThreads) k_bwd(const BwdArgs a) {
   constexpr int V8 = In::kVec;
   using St = typename In::storage;
+  pdl_trigger();
   WsPtrs ws = a.ws;
-  const long long N = ws.hdr->n_tokens;
-  float g = a.grad_loss;
-  if (a.grad_loss_dev) g *= *a.grad_loss_dev;
-  const float cscale = (N > 0) ? g / static_cast<float>(N) * a.invT : 0.0f;
 
   constexpr int kTile = kBwdTile;
   constexpr int kPer = kTile / V8 / kBwdThreads;  // vectors per thread per tile
@@ -47,8 +44,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd(const BwdArgs a) {
   // arithmetic, so each thread keeps up to 2 kPer loads in flight.
   // rows that do not train (or have a bad target) get zeros: no read
   auto reads = [&](long long row) { return a.mask[row] != 0 && !(ws.flags[row] & kFlagBad); };
-  auto load_tile = [&](long long row, int t, uint4* raw) {
-    const int nv = reads(row) ? tile_nv(t) : 0;
+  auto load_tile = [&](long long row, int t, uint4* raw, bool rd) {
+    const int nv = rd ? tile_nv(t) : 0;
     const char* zrow = static_cast<const char*>(a.logits) + row * a.ld * static_cast<long long>(sizeof(St)) +
                        static_cast<size_t>(t) * kTile * sizeof(St);
 #pragma unroll
@@ -60,12 +57,18 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd(const BwdArgs a) {
   long long row = blockIdx.x / tpr;
   int t = static_cast<int>(blockIdx.x % tpr);
   uint4 raw[kPer], nxt[kPer];
-  if (row < a.R) load_tile(row, t, raw);
+  // (the first tile's loads need nothing of the kernel before this one)
+  if (row < a.R) load_tile(row, t, raw, a.mask[row] != 0);
+  pdl_wait();
+  const long long N = ws.hdr->n_tokens;
+  float g = a.grad_loss;
+  if (a.grad_loss_dev) g *= *a.grad_loss_dev;
+  const float cscale = (N > 0) ? g / static_cast<float>(N) * a.invT : 0.0f;
   while (row < a.R) {
     long long nrow = row;
     int nt = t;
     advance(nrow, nt);
-    if (nrow < a.R) load_tile(nrow, nt, nxt);
+    if (nrow < a.R) load_tile(nrow, nt, nxt, reads(nrow));
     const int j0 = t * kTile;
     const int j1 = min(a.V, j0 + kTile);
     const char* zrow = static_cast<const char*>(a.logits) + row * a.ld * static_cast<long long>(sizeof(St));

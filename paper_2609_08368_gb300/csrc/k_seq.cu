@@ -31,6 +31,8 @@ constexpr int kWarps = kThreads / 32;
 __global__ void __launch_bounds__(kThreads) k_seq(const SeqArgs a) {
   __shared__ double s_a[kWarps], s_b[kWarps];
   __shared__ float s_out[4];  // s_i, scale * pg_i, scale * mean_w * (-A s_i) or 0, flags
+  pdl_trigger();
+  pdl_wait();
   WsPtrs ws = a.ws;
   const int i = blockIdx.x;
   if (ws.hdr->err_bits & kErrSeqlens) {  // rows cannot be attributed to trajectories

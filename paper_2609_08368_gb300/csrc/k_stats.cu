@@ -3,11 +3,20 @@
 // rollout logp| (the train/rollout divergence of Sec. 9.2) and the
 // correction ratio (Sec. 3.4), min / max ratio, and exact clip counts.
 //
-// Each block reduces a fixed strided set of rows into partial sums
+// Each block reduces a fixed strided set of rows into partial results
 // (butterfly merges in a fixed order), stores them in the workspace, and the
 // last block to finish (an atomic ticket, no waiting) merges the partials in
-// double precision in block order. The grid size depends only on the row
+// double precision in a fixed order. The grid size depends only on the row
 // count, so the scalar loss is bit-for-bit reproducible.
+//
+// Latency bounds the kernel (13 reads per row, 80 bytes, of rows the sweep has
+// just written), and the double-precision merge was most of it: 14 doubles
+// merged by every warp of the last block are some 1,400 warp instructions on
+// a unit that takes one per 16 clocks. Here each of the 16 results has its
+// own lanes, 256 threads of (result, subset of the partials), so the merge
+// is one operation per 16 partials and a fixed tree.
+#include <stddef.h>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -17,13 +26,15 @@ namespace {
 
 // Per-block partial sums: fp32 within a block (a fixed-order tree over at
 // most kStatThreads rows; its rounding is far below the statistics'
-// tolerance), exact integer counts; the last block merges the partials in
-// double precision.
+// tolerance), exact integer counts.
 struct Part {
   float v[9];  // ell, pg, k3, H, r, |r-1|, |logp-rho|, rc, |rc-1|
   float rmin, rmax;
   unsigned int c[5];  // n, clip_hi, clip_lo, dual, corr_clip
 };
+// The 16 results of a StatPart: 0..8 the sums, 9..13 the counts, then the
+// smallest and the largest ratio.
+constexpr int kCount0 = 9, kMin = 14, kMax = 15;
 
 __device__ __forceinline__ void part_zero(Part& p) {
 #pragma unroll
@@ -34,119 +45,69 @@ __device__ __forceinline__ void part_zero(Part& p) {
   for (int i = 0; i < 5; ++i) p.c[i] = 0u;
 }
 
-__device__ __forceinline__ void part_merge_shfl(Part& p, int o) {
+// The warp's results, the same in every lane.
+__device__ __forceinline__ void warp_reduce(Part& p) {
 #pragma unroll
-  for (int i = 0; i < 9; ++i) p.v[i] += __shfl_xor_sync(0xffffffffu, p.v[i], o);
-  p.rmin = fminf(p.rmin, __shfl_xor_sync(0xffffffffu, p.rmin, o));
-  p.rmax = fmaxf(p.rmax, __shfl_xor_sync(0xffffffffu, p.rmax, o));
+  for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-  for (int i = 0; i < 5; ++i) p.c[i] += __shfl_xor_sync(0xffffffffu, p.c[i], o);
-}
-
-// Block reduction in a fixed order; the result is valid in thread 0.
-__device__ void block_reduce(Part& p, Part* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int kWarps = kStatThreads / 32;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) part_merge_shfl(p, o);
-  if (lane == 0) sh[warp] = p;
-  __syncthreads();
-  if (warp == 0) {
-    if (lane < kWarps) p = sh[lane]; else part_zero(p);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part_merge_shfl(p, o);
+    for (int i = 0; i < 9; ++i) p.v[i] += __shfl_xor_sync(0xffffffffu, p.v[i], o);
+    p.rmin = fminf(p.rmin, __shfl_xor_sync(0xffffffffu, p.rmin, o));
+    p.rmax = fmaxf(p.rmax, __shfl_xor_sync(0xffffffffu, p.rmax, o));
   }
+#pragma unroll
+  for (int i = 0; i < 5; ++i) p.c[i] = __reduce_add_sync(0xffffffffu, p.c[i]);
 }
 
-__device__ __forceinline__ void to_stat(const Part& p, StatPart& s) {
-  s.s_ell = p.v[0]; s.s_pg = p.v[1]; s.s_k3 = p.v[2]; s.s_H = p.v[3]; s.s_r = p.v[4];
-  s.s_rabs = p.v[5]; s.s_lpabs = p.v[6]; s.s_rc = p.v[7]; s.s_rcabs = p.v[8];
-  s.rmin = p.rmin; s.rmax = p.rmax;
-  s.n = p.c[0]; s.n_hi = p.c[1]; s.n_lo = p.c[2]; s.n_dual = p.c[3]; s.n_corr = p.c[4];
+// Result `q` merged with another of the same kind.
+template <class T>
+__device__ __forceinline__ T merge_q(int q, T a, T b) {
+  return q < kMin ? a + b : (q == kMin ? (b < a ? b : a) : (b > a ? b : a));
+}
+__device__ __forceinline__ double none_q(int q) {
+  return q < kMin ? 0.0 : (q == kMin ? INFINITY : -INFINITY);
 }
 
-// The final merge, in double precision: one partial per thread, then a
-// fixed-order tree.
-struct Final {
-  double v[9];
-  float rmin, rmax;
-  unsigned long long c[5];
-};
-
-__device__ __forceinline__ void final_load(const StatPart* sp, Final& f) {
-  const double* d = reinterpret_cast<const double*>(sp);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) f.v[i] = __ldcg(d + i);
-  f.rmin = __ldcg(&sp->rmin);
-  f.rmax = __ldcg(&sp->rmax);
-  const unsigned long long* c = &sp->n;
-#pragma unroll
-  for (int i = 0; i < 5; ++i) f.c[i] = __ldcg(c + i);
+// One field of the statistics from the merged results f: means over the n
+// training tokens; zeros when there are none.
+__device__ __forceinline__ void write_stat(rl_loss_stats* o, int q, double f, double n) {
+  double* means = &o->loss;  // nine consecutive means, as the sums
+  int64_t* counts = &o->n_tokens;
+  if (q < kCount0) means[q] = n > 0.0 ? f * (1.0 / n) : 0.0;
+  else if (q < kMin) counts[q - kCount0] = static_cast<int64_t>(f);
+  else if (q == kMin) o->ratio_min = n > 0.0 ? static_cast<float>(f) : 0.0f;
+  else o->ratio_max = n > 0.0 ? static_cast<float>(f) : 0.0f;
 }
-
-__device__ __forceinline__ void final_zero(Final& f) {
-#pragma unroll
-  for (int i = 0; i < 9; ++i) f.v[i] = 0.0;
-  f.rmin = INFINITY;
-  f.rmax = -INFINITY;
-#pragma unroll
-  for (int i = 0; i < 5; ++i) f.c[i] = 0ull;
-}
-
-__device__ __forceinline__ void final_merge_shfl(Final& f, int o) {
-#pragma unroll
-  for (int i = 0; i < 9; ++i) f.v[i] += __shfl_xor_sync(0xffffffffu, f.v[i], o);
-  f.rmin = fminf(f.rmin, __shfl_xor_sync(0xffffffffu, f.rmin, o));
-  f.rmax = fmaxf(f.rmax, __shfl_xor_sync(0xffffffffu, f.rmax, o));
-#pragma unroll
-  for (int i = 0; i < 5; ++i) f.c[i] += __shfl_xor_sync(0xffffffffu, f.c[i], o);
-}
-
-// Means over the n = c[0] training tokens; zeros when there are none.
-__device__ rl_loss_stats stats_of(const double* v, const unsigned long long* c, float rmin,
-                                  float rmax) {
-  rl_loss_stats o;
-  const unsigned long long n = c[0];
-  const double inv = n ? 1.0 / static_cast<double>(n) : 0.0;
-  o.loss = v[0] * inv;
-  o.pg_loss_mean = v[1] * inv;
-  o.kl_mean = v[2] * inv;
-  o.entropy_mean = v[3] * inv;
-  o.ratio_mean = v[4] * inv;
-  o.ratio_absdev_mean = v[5] * inv;
-  o.logprob_absdiff_mean = v[6] * inv;
-  o.corr_ratio_mean = v[7] * inv;
-  o.corr_absdev_mean = v[8] * inv;
-  o.ratio_min = n ? rmin : 0.0f;
-  o.ratio_max = n ? rmax : 0.0f;
-  o.n_tokens = static_cast<int64_t>(n);
-  o.n_clip_hi = static_cast<int64_t>(c[1]);
-  o.n_clip_lo = static_cast<int64_t>(c[2]);
-  o.n_dual_clip = static_cast<int64_t>(c[3]);
-  o.n_corr_clip = static_cast<int64_t>(c[4]);
-  return o;
-}
+static_assert(offsetof(rl_loss_stats, corr_absdev_mean) == 8 * sizeof(double) &&
+                  offsetof(rl_loss_stats, n_corr_clip) ==
+                      offsetof(rl_loss_stats, n_tokens) + 4 * sizeof(int64_t),
+              "the means and the counts are consecutive");
 
 __global__ void __launch_bounds__(kStatThreads) k_stats(const StatArgs a) {
-  __shared__ Part sh[kStatThreads / 32];
-  __shared__ Final shf[kStatThreads / 32];
+  constexpr int kWarps = kStatThreads / 32, kSubs = kStatThreads / kStatFields;
+  __shared__ float sh_f[kWarps][kStatFields];         // the warps' sums and extremes
+  __shared__ unsigned int sh_c[kWarps][kStatFields];  // ... and counts
+  __shared__ double sh_d[kWarps][kStatFields];
   __shared__ int s_last;
   WsPtrs ws = a.ws;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_trigger();
+  pdl_wait();
   Part p;
   part_zero(p);
   const long long stride = static_cast<long long>(gridDim.x) * kStatThreads;
-  for (long long t = blockIdx.x * static_cast<long long>(kStatThreads) + threadIdx.x; t < a.R;
-       t += stride) {
-    if (!a.mask[t]) continue;
-    const uint8_t f = ws.flags[t];
-    const float r = ws.r[t], rc = ws.rc[t];
-    p.v[0] += ws.ell[t];
-    p.v[1] += ws.pg[t];
-    p.v[2] += ws.k3[t];
-    p.v[3] += ws.H[t];
+  for (long long t = blockIdx.x * static_cast<long long>(kStatThreads) + tid; t < a.R; t += stride) {
+    // every load of a row is issued at once (a masked row's values are not used)
+    const uint8_t m = a.mask[t], f = ws.flags[t];
+    const float r = ws.r[t], rc = ws.rc[t], ell = ws.ell[t], pg = ws.pg[t], k3 = ws.k3[t],
+                H = ws.H[t], logp = ws.logp[t], rho = a.rho[t];
+    if (!m) continue;
+    p.v[0] += ell;
+    p.v[1] += pg;
+    p.v[2] += k3;
+    p.v[3] += H;
     p.v[4] += r;
     p.v[5] += fabsf(r - 1.0f);
-    p.v[6] += fabsf(ws.logp[t] - a.rho[t]);
+    p.v[6] += fabsf(logp - rho);
     p.v[7] += rc;
     p.v[8] += fabsf(rc - 1.0f);
     p.rmin = fminf(p.rmin, r);
@@ -157,53 +118,87 @@ __global__ void __launch_bounds__(kStatThreads) k_stats(const StatArgs a) {
     p.c[3] += (f & kFlagDual) ? 1 : 0;
     p.c[4] += (f & kFlagCorrClip) ? 1 : 0;
   }
-  block_reduce(p, sh);
-  if (threadIdx.x == 0) {
-    to_stat(p, ws.parts[blockIdx.x]);
-    __threadfence();
-    const unsigned int ticket = atomicAdd(&ws.hdr->ticket, 1u);
-    s_last = (ticket == gridDim.x - 1) ? 1 : 0;
+  warp_reduce(p);
+  if (lane == 0) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) sh_f[warp][i] = p.v[i];
+    sh_f[warp][kMin] = p.rmin;
+    sh_f[warp][kMax] = p.rmax;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) sh_c[warp][kCount0 + i] = p.c[i];
   }
   __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-
-  // Last block: merge the partials in block order (one per thread, then a tree).
-  Final fin;
-  if (static_cast<int>(threadIdx.x) < static_cast<int>(gridDim.x)) final_load(&ws.parts[threadIdx.x], fin);
-  else final_zero(fin);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // the block's results: thread q < 16 merges the warps' result q, in order
+  const int q = tid & (kStatFields - 1);
+  const bool is_count = q >= kCount0 && q < kMin;
+  double mine = 0.0;
+  if (tid < kStatFields) {
+    if (is_count) {
+      unsigned int c = 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) final_merge_shfl(fin, o);
-  if (lane == 0) shf[warp] = fin;
-  __syncthreads();
-  if (warp == 0) {
-    if (lane < kStatThreads / 32) fin = shf[lane]; else final_zero(fin);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) final_merge_shfl(fin, o);
-  }
-  if (threadIdx.x == 0) {
-    if (a.part_out) {
-      rl_loss_partials p;
-      for (int i = 0; i < 9; ++i) p.sum[i] = fin.v[i];
-      for (int i = 0; i < 5; ++i) p.count[i] = static_cast<double>(fin.c[i]);
-      p.max[0] = fin.c[0] ? -static_cast<double>(fin.rmin) : -INFINITY;
-      p.max[1] = fin.c[0] ? static_cast<double>(fin.rmax) : -INFINITY;
-      *a.part_out = p;
+      for (int w = 0; w < kWarps; ++w) c += sh_c[w][q];
+      mine = static_cast<double>(c);
     } else {
-      *a.out = stats_of(fin.v, fin.c, fin.rmin, fin.rmax);
+      float v = sh_f[0][q];
+#pragma unroll
+      for (int w = 1; w < kWarps; ++w) v = merge_q(q, v, sh_f[w][q]);
+      mine = static_cast<double>(v);
     }
-    ws.hdr->ticket = 0;
+  }
+  if (gridDim.x > 1) {
+    if (warp == 0) {
+      if (lane < kStatFields) {
+        ws.parts[blockIdx.x].f[lane] = mine;
+        __threadfence();
+      }
+      __syncwarp();
+      if (lane == 0) {
+        const unsigned int ticket = atomicAdd(&ws.hdr->ticket, 1u);
+        s_last = (ticket == gridDim.x - 1) ? 1 : 0;
+      }
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // Last block: thread (sub, q) merges result q of the partials sub,
+    // sub + 16, ... in order, then the 16 subsets in a fixed order.
+    const int sub = tid / kStatFields;
+    double v = none_q(q);
+    for (int b = sub; b < static_cast<int>(gridDim.x); b += kSubs)
+      v = merge_q(q, v, __ldcg(&ws.parts[b].f[q]));
+    v = merge_q(q, v, __shfl_xor_sync(0xffffffffu, v, kStatFields));
+    if (lane < kStatFields) sh_d[warp][q] = v;
+    __syncthreads();
+    if (tid < kStatFields) {
+      mine = sh_d[0][q];
+#pragma unroll
+      for (int w = 1; w < kWarps; ++w) mine = merge_q(q, mine, sh_d[w][q]);
+    }
+    if (tid == 0) ws.hdr->ticket = 0;
+  }
+  if (warp != 0) return;
+  const double n = __shfl_sync(0xffffffffu, mine, kCount0);
+  if (lane >= kStatFields) return;
+  if (a.part_out) {
+    if (q < kCount0) a.part_out->sum[q] = mine;
+    else if (q < kMin) a.part_out->count[q - kCount0] = mine;
+    else if (q == kMin) a.part_out->max[0] = n > 0.0 ? -mine : -INFINITY;
+    else a.part_out->max[1] = n > 0.0 ? mine : -INFINITY;
+  } else {
+    write_stat(a.out, q, mine, n);
   }
 }
 
-// The statistics of a sharded call from its shards' combined partials.
+// The statistics of a sharded call from its shards' combined partials, one
+// result per lane.
 __global__ void k_finish(const FinishArgs a) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const rl_loss_partials p = *a.part;
-  unsigned long long c[5];
-  for (int i = 0; i < 5; ++i) c[i] = static_cast<unsigned long long>(p.count[i]);
-  *a.out = stats_of(p.sum, c, static_cast<float>(-p.max[0]), static_cast<float>(p.max[1]));
+  const int q = threadIdx.x;
+  if (q >= kStatFields || blockIdx.x != 0) return;
+  const double n = a.part->count[0];
+  const double f = q < kCount0 ? a.part->sum[q]
+                               : (q < kMin ? a.part->count[q - kCount0]
+                                           : (q == kMin ? -a.part->max[0] : a.part->max[1]));
+  write_stat(a.out, q, f, n);
 }
 
 }  // namespace

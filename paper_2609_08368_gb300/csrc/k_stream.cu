@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
   constexpr int V8 = In::kVec;
   constexpr int P = V8 / 2;
   extern __shared__ __align__(128) unsigned char smem[];
+  pdl_trigger();
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   const int NS = a.n_slots;
@@ -454,10 +455,7 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
   }
 
   // -------------------------------------------------------------- consumers
-  const long long N = ws.hdr->n_tokens;
-  float g = a.grad_loss;
-  if (a.grad_loss_dev) g *= *a.grad_loss_dev;
-  const float cscale = (N > 0) ? g / static_cast<float>(N) * a.s.invT : 0.0f;
+  float cscale = 0.0f;  // (thread 0, from its first row's epilogue on)
   const float2 k2 = make_float2(k, k);
   // the sampled token's dLogit of the previous row, written after the next
   // barrier (so after every store of that row)
@@ -510,7 +508,7 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
       rho = a.rho[row];
       if (a.q) q = a.q[row];
       if (a.old) old = a.old[row];
-      A = ws.a_row[row];
+      if (i > 0) A = ws.a_row[row];
       msk = trains ? 1 : 0;
       yok = y >= 0;
       if (yok && y >= my_tail0) zy = In::load1(grow, y);
@@ -583,6 +581,16 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
       const float tt = fmaf(z, k, -t.m), x = ex2(tt);
       t.s += x;
       t.u = fmaf(x, tt, t.u);
+    }
+
+    if (i == 0 && tid == 0) {
+      // the advantage kernel's results: it may still be running until here
+      pdl_wait();
+      A = ws.a_row[row];
+      const long long N = ws.hdr->n_tokens;
+      float g = a.grad_loss;
+      if (a.grad_loss_dev) g *= *a.grad_loss_dev;
+      cscale = (N > 0) ? g / static_cast<float>(N) * a.s.invT : 0.0f;
     }
 
     // ---------------- merge

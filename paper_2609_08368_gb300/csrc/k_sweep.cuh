@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep(const SweepArgs 
   constexpr int P = V8 / 2;
   constexpr int kWarps = kThreads / 32;
   extern __shared__ __align__(128) unsigned char smem[];
+  pdl_trigger();
   const int tid = threadIdx.x;
   const int C = static_cast<int>(cluster_nctarank());
   const int crank = static_cast<int>(cluster_ctarank());
@@ -194,10 +195,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep(const SweepArgs 
 
   WsPtrs ws = a.ws;
   uint32_t* err = &ws.hdr->err_bits;
-  const long long N = ws.hdr->n_tokens;
-  float g = a.grad_loss;
-  if (a.grad_loss_dev) g *= *a.grad_loss_dev;
-  const float cscale = (N > 0) ? g / static_cast<float>(N) * a.s.invT : 0.0f;
+  float cscale = 0.0f;  // (thread 0, from its first row's epilogue on)
 
   if (tid == 0) {
     for (int s = 0; s < S; ++s) mbar_init(smem_u32(&bars[s]), 1);
@@ -271,7 +269,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep(const SweepArgs 
       rho = a.rho[row];
       if (a.q) q = a.q[row];
       if (a.old) old = a.old[row];
-      A = ws.a_row[row];
+      if (it > 0) A = ws.a_row[row];
       msk = a.mask[row];
     }
     // top-K OPD candidates (warp 0): this row's ids and teacher values
@@ -343,6 +341,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep(const SweepArgs 
       topk_gather<In>(tk, grow + static_cast<size_t>(vec_elems) * sizeof(St), lo + vec_elems, lo + cnt);
       const int c0 = lo, c1 = lo + cnt;
       tkp = topk_part(tk, tk_row, tid, a.s.invT, k, [c0, c1](int id) { return id >= c0 && id < c1; });
+    }
+    if (it == 0 && tid == 0) {
+      // the advantage kernel's results: it may still be running until here
+      pdl_wait();
+      A = ws.a_row[row];
+      const long long N = ws.hdr->n_tokens;
+      float g = a.grad_loss;
+      if (a.grad_loss_dev) g *= *a.grad_loss_dev;
+      cscale = (N > 0) ? g / static_cast<float>(N) * a.s.invT : 0.0f;
     }
     t = block_merge<kWarps>(t, red);
 

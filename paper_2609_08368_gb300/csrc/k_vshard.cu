@@ -33,6 +33,7 @@ namespace {
 constexpr float kLn2f = 0.69314718055994531f;
 
 __global__ void __launch_bounds__(kMergeThreads) k_vmerge(const MergeArgs a) {
+  pdl_trigger();  // (the first kernel of its call)
   WsPtrs ws = a.ws;
   uint32_t* err = &ws.hdr->err_bits;
   const long long V_total = a.col_starts[a.n_shards];

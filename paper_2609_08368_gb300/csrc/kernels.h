@@ -11,7 +11,12 @@ namespace milesloss {
 constexpr int kMaxStages = 4;
 constexpr int kMaxCluster = 8;
 constexpr uint32_t kBulkChunk = 16384;    // bytes per cp.async.bulk
-constexpr int kAdvThreads = 1024;
+constexpr int kAdvThreads = 512;
+// CTAs of the advantage kernel (one cluster). With 1 / 4 / 8: 512 trajectories of
+// 64 rows x 32,768 fp32 1,426 / 1,337 / 1,327 us a call, 128 x 128 rows x 20,480
+// (forward) 144 / 131 / 127, 16,384 rows x 151,936 1,548 / 1,535 / 1,533; the same to
+// 1 us on 2,048 rows x 4,096.
+constexpr int kAdvCluster = 8;
 constexpr int kBwdThreads = 256;
 // k_stream's block: cw consumer warps (16 with one CTA per SM, 8 with two, 4
 // with four),
@@ -106,8 +111,9 @@ struct AdvArgs {
   int normalize_std, unbiased_std;
   float std_floor;
   int estimator;   // rl_estimator
-  int smem_traj;   // trajectory tables (cu_seqlens, group ids, rewards, counts,
-                   // advantages) staged in shared memory
+  int smem_traj;   // trajectory tables (cu_seqlens, group ids, rewards) staged in
+                   // shared memory
+  int groups_done; // k_groups has computed the group statistics
   float* advantages;   // may be null
   int* group_sizes;    // may be null
   WsPtrs ws;
@@ -216,9 +222,12 @@ const void* bwd_kernel(rl_dtype in, rl_dtype out);
 const void* adv_kernel();
 const void* groups_kernel();  // one 32-thread block per group (grid-stride)
 constexpr int kMaxGroupBlocks = 65535;
-// Up to this many groups, k_advantages computes the group statistics itself
-// (a launch costs more than their double arithmetic on one SM).
-constexpr int kInlineGroups = 8;
+// k_advantages computes the group statistics itself unless its cluster's
+// warps (128) would scan the trajectories for several hundred steps of 32
+// each: then k_groups spreads the groups over the whole GPU first.
+inline bool group_kernel_pays(long long n_groups, long long n_traj) {
+  return n_groups * n_traj > (1LL << 20);
+}
 const void* seq_kernel();
 const void* merge_kernel();   // vocabulary-sharded calls: k_vmerge
 const void* stats_kernel();
