@@ -192,8 +192,12 @@ rl_status rl_loss_workspace_size(int64_t n_rows, int32_t n_traj, int32_t n_group
  *                    holds the logits that scored targets[t] (already shifted
  *                    by the caller); only the first `vocab` columns are read.
  *                    Rows whose start is 16-byte aligned (ld * element size a
- *                    multiple of 16 and a 16-byte aligned base) take the
- *                    fast bulk-copy path; any other layout is still correct.
+ *                    multiple of 16 and a 16-byte aligned base) are fastest;
+ *                    any other layout is correct (bf16 rows are then copied
+ *                    in the 16-byte granules they touch, so the neighbours'
+ *                    bytes in a row's first and last granule are fetched too,
+ *                    never bytes outside the rows; fp32 rows go element by
+ *                    element).
  *  targets           [n_rows] int32 sampled token ids, in [0, vocab)
  *  rollout_logprobs  [n_rows] fp32 log-probs the rollout engine reported
  *  ref_logprobs      [n_rows] fp32 reference-policy log-probs, or NULL
@@ -506,7 +510,7 @@ const char* rl_status_string(rl_status status);
  * every field to -1. A forced value outside the compiled shapes makes later
  * calls return RL_ERR_UNSUPPORTED before anything is enqueued.
  *  sweep_kernel         0 = the cluster kernel, 1 = the streaming kernel
- *                       (16-byte aligned rows only)
+ *                       (not unaligned fp32 logits)
  *  cluster_size         1, 2, 4 or 8 CTAs per row (cluster kernel)
  *  cluster_stages       1..4 ring stages (cluster kernel)
  *  cluster_threads      256 or 512 threads per CTA (cluster kernel)

@@ -430,8 +430,8 @@ rl_status launch_bwd(const Common& c, const GradOut& go, const WsPtrs& ws, cudaS
   b.V = static_cast<int>(c.V);
   b.tiles_per_row = static_cast<int>((c.V + kBwdTile - 1) / kBwdTile);
   b.n_tiles = c.R * b.tiles_per_row;
-  b.in_vec = aligned16(c.logits) && ((c.ld * elem_size(c.dt)) % 16 == 0);
-  b.out_vec = aligned16(go.dl) && ((go.ld_out * elem_size(go.dt)) % 16 == 0);
+  const bool unal = !aligned16(c.logits) || (c.ld * elem_size(c.dt)) % 16 != 0 ||
+                    !aligned16(go.dl) || (go.ld_out * elem_size(go.dt)) % 16 != 0;
   b.targets = c.targets;
   b.mask = c.mask;
   b.dlogits = go.dl;
@@ -445,7 +445,7 @@ rl_status launch_bwd(const Common& c, const GradOut& go, const WsPtrs& ws, cudaS
   b.ws = ws;
   // one wave of resident blocks (grid-stride over the tiles): a second,
   // partial wave would run with fewer loads in flight
-  const void* fn = bwd_kernel(c.dt, go.dt);
+  const void* fn = bwd_kernel(c.dt, go.dt, unal);
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBwdThreads, 0) != cudaSuccess)
     return RL_ERR_CUDA;
@@ -580,21 +580,32 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
   const size_t es = elem_size(c.dt);
   const bool in_bulk = aligned16(c.logits) && ((c.ld * es) % 16 == 0);
   const bool out_vec = grad && aligned16(go->dl) && ((go->ld_out * elem_size(go->dt)) % 16 == 0);
+  const bool unal = !in_bulk || (grad && !out_vec);
   const rl_launch_overrides ov = current_overrides();
   const unsigned long long stall =
       ov.stall_first_wait_ns > 0 ? static_cast<unsigned long long>(ov.stall_first_wait_ns) : 0ull;
-  if (c.R > 0 &&
-      use_stream(c.V * static_cast<long long>(es), static_cast<int>(es), in_bulk, grad, sc.topk > 0, ov)) {
-    StreamPlan sp;
+  const long long row_bytes = c.V * static_cast<long long>(es);
+  // (unaligned rows whose ring, forced by an override, has no room for the
+  // slots' padding: the cluster kernel)
+  StreamPlan sp;
+  bool stream = c.R > 0 && use_stream(row_bytes, static_cast<int>(es), in_bulk, unal, grad,
+                                      sc.topk > 0, ov);
+  if (stream && unal) {
+    st = plan_stream(dev, sc.topk ? kTopKSmem : 0, row_bytes, static_cast<int>(es), grad,
+                     sc.topk > 0, unal, f.part_rows == nullptr, ov, &sp);
+    if (st == RL_ERR_UNSUPPORTED) stream = false;
+    else if (st != RL_OK) return st;
+  }
+  if (c.R > 0 && stream) {
     const void* fn = nullptr;
     int ctas = 0;  // resident CTAs, or clusters of sp.cluster CTAs
     int threads = 0;
     rl_launch_overrides pov = ov;
     for (;;) {
-      st = plan_stream(dev, sc.topk ? kTopKSmem : 0, c.V * static_cast<long long>(es),
-                       static_cast<int>(es), grad, sc.topk > 0, f.part_rows == nullptr, pov, &sp);
+      st = plan_stream(dev, sc.topk ? kTopKSmem : 0, row_bytes, static_cast<int>(es), grad,
+                       sc.topk > 0, unal, f.part_rows == nullptr, pov, &sp);
       if (st != RL_OK) return st;
-      fn = stream_kernel(c.dt, grad ? go->dt : c.dt, grad, sc.topk > 0, sp.cw, sp.cluster > 1);
+      fn = stream_kernel(c.dt, grad ? go->dt : c.dt, grad, sc.topk > 0, unal, sp.cw, sp.cluster > 1);
       if (!fn) return RL_ERR_UNSUPPORTED;
       st = set_smem(fn, dev, sp.smem);
       if (st != RL_OK) return st;
@@ -619,7 +630,6 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     ta.n_hold = sp.hold;
     ta.split_first = sp.split_first;
     ta.prefetch = sp.prefetch;
-    ta.out_vec = out_vec;
     ta.slice_vec = sp.slice_vec;
     ta.targets = c.targets;
     ta.rho = fr.rho;

@@ -630,16 +630,16 @@ __device__ __forceinline__ void topk_prefetch(TopKBuf* buf, const int* ids, cons
 // columns [col0, col0 + V) of a vocabulary of V_total (col0 = 0, V_total = V
 // unless the call is a vocabulary shard): -1 for a candidate in another
 // shard's columns; an id outside [0, V_total) marks the row bad.
-__device__ __forceinline__ TopKLane topk_ids(const TopKBuf* buf, int col0, int V, int V_total,
+__device__ __forceinline__ TopKLane topk_ids(const int* ids, int col0, int V, int V_total,
                                              int K, int lane) {
   TopKLane c{-1, -1, 0.0f, 0.0f, false};
   if (lane < K) {
-    const int id = buf->ids[lane];
+    const int id = ids[lane];
     if (id < 0 || id >= V_total) c.bad = true;
     else if (id - col0 >= 0 && id - col0 < V) c.id0 = id - col0;
   }
   if (lane + 32 < K) {
-    const int id = buf->ids[lane + 32];
+    const int id = ids[lane + 32];
     if (id < 0 || id >= V_total) c.bad = true;
     else if (id - col0 >= 0 && id - col0 < V) c.id1 = id - col0;
   }
@@ -676,7 +676,7 @@ __device__ __forceinline__ TopKPart topk_merge_all(const float4* parts, int n) {
 // The warp's part over its lanes' candidates whose ids satisfy `mine`
 // (fixed-order butterfly; every lane ends with it); k = log2(e) / T.
 template <class Mine>
-__device__ __forceinline__ TopKPart topk_part(const TopKLane& c, const TopKBuf* buf, int lane,
+__device__ __forceinline__ TopKPart topk_part(const TopKLane& c, const float* teacher, int lane,
                                               float invT, float k, Mine mine) {
   const bool u0 = c.id0 >= 0 && mine(c.id0), u1 = c.id1 >= 0 && mine(c.id1);
   const int bad = __any_sync(0xffffffffu, c.bad) ? 1 : 0;
@@ -687,8 +687,8 @@ __device__ __forceinline__ TopKPart topk_part(const TopKLane& c, const TopKBuf* 
   if (M == -INFINITY) return TopKPart{-INFINITY, 0.0f, 0.0f, bad};
   const float w0 = u0 ? ex2(t0 - M) : 0.0f, w1 = u1 ? ex2(t1 - M) : 0.0f;
   float sw = w0 + w1;
-  float acc = (u0 ? w0 * fmaf(c.z0, invT, -buf->teacher[lane]) : 0.0f) +
-              (u1 ? w1 * fmaf(c.z1, invT, -buf->teacher[lane + 32]) : 0.0f);
+  float acc = (u0 ? w0 * fmaf(c.z0, invT, -teacher[lane]) : 0.0f) +
+              (u1 ? w1 * fmaf(c.z1, invT, -teacher[lane + 32]) : 0.0f);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     sw += __shfl_xor_sync(0xffffffffu, sw, o);

@@ -336,11 +336,11 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep(const SweepArgs 
     // shared memory, past its whole vectors from global memory
     TopKPart tkp{-INFINITY, 0.0f, 0.0f, 0};
     if (topk && tid < 32) {
-      TopKLane tk = topk_ids(tk_row, static_cast<int>(a.col0), a.V, a.vocab_total, a.s.topk, tid);
+      TopKLane tk = topk_ids(tk_row->ids, static_cast<int>(a.col0), a.V, a.vocab_total, a.s.topk, tid);
       if (have) topk_gather<In>(tk, sb, lo, lo + vec_elems);
       topk_gather<In>(tk, grow + static_cast<size_t>(vec_elems) * sizeof(St), lo + vec_elems, lo + cnt);
       const int c0 = lo, c1 = lo + cnt;
-      tkp = topk_part(tk, tk_row, tid, a.s.invT, k, [c0, c1](int id) { return id >= c0 && id < c1; });
+      tkp = topk_part(tk, tk_row->teacher, tid, a.s.invT, k, [c0, c1](int id) { return id >= c0 && id < c1; });
     }
     if (it == 0 && tid == 0) {
       // the advantage kernel's results: it may still be running until here

@@ -71,7 +71,6 @@ struct StreamArgs {
   int n_hold;       // last chunks of a row that pass B reads from shared memory (<= n_slots)
   int split_first;  // 1: the first chunk takes the ragged remainder (rounded up to 128 bytes)
   int prefetch;     // bytes of the next row to ask L2 for once a row's first pass is issued
-  int out_vec;      // dLogits rows are 16-byte aligned: vector stores
   int slice_vec;    // launched in clusters (one per row): whole vectors of a row per CTA, a
                     // multiple of 8 (the cluster's last CTA may take fewer, or none)
   const int* targets;
@@ -156,7 +155,6 @@ struct BwdArgs {
   int V;
   int tiles_per_row;
   long long n_tiles;
-  int in_vec, out_vec;
   const int* targets;
   const uint8_t* mask;
   void* dlogits;
@@ -199,7 +197,10 @@ const void* sweep_kernel(rl_dtype in, rl_dtype out, bool grad, int threads, bool
 const void* sweep_kernel_topk(rl_dtype in, rl_dtype out, bool grad, int threads);
 // clu: the instantiation that runs in clusters of CTAs per row (fused
 // calls without top-K only; nullptr otherwise)
-const void* stream_kernel(rl_dtype in, rl_dtype out, bool grad, bool topk, int cw, bool clu);
+// unal: the instantiations for rows that do not all start on a 16-byte boundary
+const void* stream_kernel(rl_dtype in, rl_dtype out, bool grad, bool topk, bool unal, int cw,
+                          bool clu);
+const void* stream_kernel_unal(rl_dtype in, rl_dtype out, bool grad, bool topk, int cw, bool clu);
 
 // The process-wide launch-plan overrides set by rl_set_launch_overrides (a
 // copy; every field -1 when none are set).
@@ -210,15 +211,16 @@ rl_status status_of_bits(uint32_t bits);
 // The streaming kernel's launch plan (k_stream.cu, from the pure plan in
 // stream_plan.h): whether rows of row_bytes go to it, and its ring of
 // shared-memory slots.
-bool use_stream(long long row_bytes, int es, bool in_bulk, bool grad, bool topk,
+// (unal: the rows of the logits or of dLogits do not all start on a 16-byte boundary)
+bool use_stream(long long row_bytes, int es, bool in_bulk, bool unal, bool grad, bool topk,
                 const rl_launch_overrides& ov);
 // extra: shared memory beyond the ring and the fixed scratch (kTopKSmem with
 // top-K OPD on, else 0); the ring's shape depends on the row length and on
 // whether the call writes dLogits
 // (can_cluster: the call may run a row over a cluster of CTAs)
 rl_status plan_stream(int dev, int extra, long long row_bytes, int es, bool grad, bool topk,
-                      bool can_cluster, const rl_launch_overrides& ov, StreamPlan* out);
-const void* bwd_kernel(rl_dtype in, rl_dtype out);
+                      bool unal, bool can_cluster, const rl_launch_overrides& ov, StreamPlan* out);
+const void* bwd_kernel(rl_dtype in, rl_dtype out, bool unal);
 const void* adv_kernel();
 const void* groups_kernel();  // one 32-thread block per group (grid-stride)
 constexpr int kMaxGroupBlocks = 65535;

@@ -13,14 +13,14 @@ namespace milesloss {
 
 constexpr int kSweepSmemExtra = 1024;  // mbarriers + exchange + reduction scratch
 constexpr int kMaxSlots = 16;          // ring slots of k_stream
+constexpr int kUnalPad = 16;           // a slot's bytes past its chunk when rows are unaligned
 
 // Which kernel sweeps rows of row_bytes, and with how many streaming CTAs per
 // SM: 0 = the cluster kernel, 1 = one streaming CTA per SM (sixteen consumer
 // warps, the whole shared memory for its ring), 2 or 4 = that many CTAs per SM
 // (eight or four consumer warps, a half or a quarter of the shared memory),
 // so that one CTA's per-row merge and epilogue overlap the other CTAs'
-// passes. Rows must start 16-byte aligned to stream (else the cluster
-// kernel). Measured on GB300 (fractions of the copy peak, A/B on one box,
+// passes. The table is for rows that start 16-byte aligned (others: below). Measured on GB300 (fractions of the copy peak, A/B on one box,
 // bf16 and fp32 rows):
 //   fused: rows of 192-310 KB one CTA 0.966-0.984 against 0.939-0.959 in
 //   clusters; 56-80 KB rows two CTAs 0.956-1.00 against 0.91-0.94; 20-56 KB
@@ -56,15 +56,25 @@ inline bool fp32_mid_row(long long row_bytes, int es, bool grad, bool topk) {
 // +2.9 / +1.8 / +1.7 / +1.3 % on one box, 144 / 160 KB +4.1 / +3.5 % on
 // another. (bf16 rows of that length: from 3 % ahead on one box to 2 % behind
 // on another, where the clusters ran 0.96-0.99; they stay in clusters.)
-inline bool halves_row(long long row_bytes, int es, bool grad) {
+inline bool halves_row(long long row_bytes, int es, bool grad, bool unal) {
   constexpr long long KB = 1024;
-  return grad && es == 4 && row_bytes >= 136 * KB && row_bytes < 192 * KB;
+  return grad && (es == 4 || unal) && row_bytes >= 136 * KB && row_bytes < 192 * KB;
 }
 
-inline int stream_ctas(long long row_bytes, int es, bool grad, bool topk) {
+// unal: rows that do not all start on a 16-byte boundary. The cluster kernel
+// reads and writes those element by element (4,096 x 45,003 bf16: 937 us
+// against 135), so every length streams: those the table above gives to the
+// cluster kernel with the CTAs per SM that came closest to it there.
+inline int stream_ctas(long long row_bytes, int es, bool grad, bool topk, bool unal = false) {
   constexpr long long KB = 1024;
+  if (unal) {
+    const int n = stream_ctas(row_bytes, es, grad, topk);
+    if (n > 0) return n;
+    if (grad && row_bytes >= 136 * KB) return 1;
+    return (topk || row_bytes > 56 * KB) ? 2 : 4;
+  }
   if (grad) {
-    if (row_bytes >= 192 * KB || halves_row(row_bytes, es, grad)) return 1;
+    if (row_bytes >= 192 * KB || halves_row(row_bytes, es, grad, false)) return 1;
     if (fp32_mid_row(row_bytes, es, grad, topk)) return 2;
     if (row_bytes > 56 * KB && row_bytes <= 80 * KB) return 2;
     if (!topk && row_bytes >= 20 * KB && row_bytes <= 56 * KB) return 4;
@@ -141,14 +151,15 @@ inline int slice_vectors(long long row_vec, int C) {
 // fixed scratch (with top-K OPD on, its candidate buffers) and the
 // overrides; false when a forced value does not fit.
 inline bool plan_ring(long long row_bytes, int es, bool grad, bool topk, const SmemLimits& lim,
-                      int extra, const rl_launch_overrides& ov, StreamPlan* out) {
+                      int extra, const rl_launch_overrides& ov, StreamPlan* out,
+                      bool unal = false) {
   const int per = ov.stream_ctas_per_sm > 0 ? ov.stream_ctas_per_sm
-                                            : std::max(1, stream_ctas(row_bytes, es, grad, topk));
+                                            : std::max(1, stream_ctas(row_bytes, es, grad, topk, unal));
   if (per != 1 && per != 2 && per != 4) return false;
   const bool lng = grad && row_bytes >= kLongRowBytes;
   const int budget = per > 1 ? std::min(lim.optin, lim.per_sm / per - lim.reserved) : lim.optin;
   int chunk_d = lng ? 75776 : 114688, hold_d = lng ? 2 : 1, split_d = lng ? 1 : 0;
-  if (per == 1 && halves_row(row_bytes, es, grad)) {
+  if (per == 1 && halves_row(row_bytes, es, grad, unal)) {
     chunk_d = static_cast<int>(((row_bytes + 1) / 2 + 127) / 128 * 128);
     hold_d = 0;
     split_d = 1;
@@ -168,7 +179,8 @@ inline bool plan_ring(long long row_bytes, int es, bool grad, bool topk, const S
   }
   const int chunk = ov.stream_chunk_bytes > 0 ? ov.stream_chunk_bytes : chunk_d;
   if (chunk < 1024 || chunk > 131072 || chunk % 128) return false;
-  int slots = (budget - kSweepSmemExtra - extra) / chunk;
+  const int slot = chunk + (unal ? kUnalPad : 0);
+  int slots = (budget - kSweepSmemExtra - extra) / slot;
   if (slots > kMaxSlots) slots = kMaxSlots;
   if (ov.stream_slots > 0) {
     if (ov.stream_slots > slots) return false;
@@ -182,7 +194,7 @@ inline bool plan_ring(long long row_bytes, int es, bool grad, bool topk, const S
   out->hold = hold;
   out->split_first = ov.stream_split_first >= 0 ? ov.stream_split_first : split_d;
   out->prefetch = ov.stream_prefetch_bytes >= 0 ? ov.stream_prefetch_bytes : 0;
-  out->smem = slots * chunk + kSweepSmemExtra + extra;
+  out->smem = slots * slot + kSweepSmemExtra + extra;
   out->cw = 16 / per;
   out->cluster = 1;
   out->slice_vec = 0;
@@ -199,18 +211,19 @@ inline bool plan_ring(long long row_bytes, int es, bool grad, bool topk, const S
 // when a forced value does not fit.
 inline bool plan_stream_rows(long long row_bytes, int es, bool grad, bool topk, bool can_cluster,
                              const SmemLimits& lim, int extra, const rl_launch_overrides& ov,
-                             StreamPlan* out) {
+                             StreamPlan* out, bool unal = false) {
   const bool can = can_cluster && grad && !topk;
   int C = 1;
   if (can && ov.stream_cluster > 0) C = ov.stream_cluster;
   else if (can && ov.stream_ctas_per_sm <= 1) C = stream_cluster(row_bytes, es, grad, topk);
-  if (C == 1) return plan_ring(row_bytes, es, grad, topk, lim, extra, ov, out);
+  if (C == 1) return plan_ring(row_bytes, es, grad, topk, lim, extra, ov, out, unal);
   if (C != 2 && C != 4 && C != 8) return false;
   if (ov.stream_ctas_per_sm > 1) return false;
   const int sv = slice_vectors(row_bytes / 16, C);
   rl_launch_overrides one = ov;
   one.stream_ctas_per_sm = 1;
-  if (!plan_ring(static_cast<long long>(sv) * 16, es, grad, topk, lim, extra, one, out)) return false;
+  if (!plan_ring(static_cast<long long>(sv) * 16, es, grad, topk, lim, extra, one, out, unal))
+    return false;
   out->cluster = C;
   out->slice_vec = sv;
   return true;
