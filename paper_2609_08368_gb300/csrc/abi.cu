@@ -596,7 +596,42 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     if (st == RL_ERR_UNSUPPORTED) stream = false;
     else if (st != RL_OK) return st;
   }
-  if (c.R > 0 && stream) {
+  if (c.R > 0 && use_short(row_bytes, unal, ov)) {
+    int warps = 0, nv = 0, sms = 0;
+    short_shape(row_bytes / 16, &warps, &nv);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return RL_ERR_CUDA;
+    ShortArgs ha;
+    ha.logits = c.logits;
+    ha.ld = c.ld;
+    ha.R = c.R;
+    ha.V = static_cast<int>(c.V);
+    ha.first_wave = 4 * sms;
+    ha.targets = c.targets;
+    ha.rho = fr.rho;
+    ha.q = fr.q;
+    ha.old = fr.old;
+    ha.mask = c.mask;
+    ha.out_logp = fr.out_logp;
+    ha.out_H = fr.out_H;
+    ha.dlogits = grad ? go->dl : nullptr;
+    ha.ld_out = grad ? go->ld_out : 0;
+    ha.grad_loss = grad ? go->g : 0.0f;
+    ha.grad_loss_dev = grad ? go->g_dev : nullptr;
+    ha.s = sc;
+    ha.ws = ws;
+    ha.col0 = f.col0;
+    ha.vocab_total = f.vocab_total > 0 ? f.vocab_total : ha.V;
+    ha.part_rows = shift(f.part_rows, 2 * r0);
+    const long long rows = kShortThreads / (32 * warps);
+    record(t_ev_begin, s);
+    st = launch(short_kernel(c.dt, grad ? go->dt : c.dt, grad, sc.topk > 0, warps, nv),
+                dim3(static_cast<unsigned>((c.R + rows - 1) / rows)), dim3(kShortThreads), 0, 1, s,
+                &ha, pdl);
+    record(t_ev_end, s);
+    if (st != RL_OK) return st;
+    pdl = overlap;
+  } else if (c.R > 0 && stream) {
     const void* fn = nullptr;
     int ctas = 0;  // resident CTAs, or clusters of sp.cluster CTAs
     int threads = 0;

@@ -22,6 +22,7 @@ constexpr int kBwdThreads = 256;
 // with four),
 // the producer warp and, with top-K OPD, the top-K warp
 constexpr int stream_threads(bool topk, int cw) { return cw * 32 + (topk ? 64 : 32); }
+constexpr int kShortThreads = 128;
 constexpr int kSeqThreads = 256;
 constexpr int kAdvSmemBytes = 48 * 1024;  // on-chip trajectory tables when they fit
 constexpr int kTopKSmem = 2 * (2 * kMaxTopK * 4);  // two rows of top-K ids + teacher values
@@ -88,6 +89,29 @@ struct StreamArgs {
   WsPtrs ws;
   unsigned long long stall_ns;  // test hook, as in SweepArgs (the consumers' first wait)
   long long col0;               // vocabulary-sharded calls, as in SweepArgs
+  int vocab_total;
+  float4* part_rows;
+};
+
+struct ShortArgs {  // k_short; the fields of SweepArgs that it needs
+  const void* logits;
+  long long ld, R;
+  int V;
+  int first_wave;   // CTAs that may start before the advantage kernel has finished
+  const int* targets;
+  const float* rho;
+  const float* q;
+  const float* old;
+  const uint8_t* mask;
+  float* out_logp;
+  float* out_H;
+  void* dlogits;
+  long long ld_out;
+  float grad_loss;
+  const float* grad_loss_dev;
+  LossScalars s;
+  WsPtrs ws;
+  long long col0;
   int vocab_total;
   float4* part_rows;
 };
@@ -195,6 +219,9 @@ constexpr int kBwdTile = kBwdThreads * 8 * 4;  // elements of one row per backwa
 // carry none of its code)
 const void* sweep_kernel(rl_dtype in, rl_dtype out, bool grad, int threads, bool topk);
 const void* sweep_kernel_topk(rl_dtype in, rl_dtype out, bool grad, int threads);
+// k_short: warps per row and vectors per lane as short_shape gives them
+const void* short_kernel(rl_dtype in, rl_dtype out, bool grad, bool topk, int warps, int nv);
+const void* short_kernel_topk(rl_dtype in, rl_dtype out, bool grad, int warps, int nv);
 // clu: the instantiation that runs in clusters of CTAs per row (fused
 // calls without top-K only; nullptr otherwise)
 // unal: the instantiations for rows that do not all start on a 16-byte boundary

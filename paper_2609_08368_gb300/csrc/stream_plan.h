@@ -87,6 +87,25 @@ inline int stream_ctas(long long row_bytes, int es, bool grad, bool topk, bool u
   return 0;
 }
 
+// Rows of up to kShortRowBytes that start 16-byte aligned (logits and
+// dLogits): k_short, with the row in registers, unless an override asks for a
+// launch shape of the other kernels.
+constexpr long long kShortRowBytes = 20 * 1024;
+inline bool use_short(long long row_bytes, bool unal, const rl_launch_overrides& ov) {
+  const bool forced = ov.sweep_kernel >= 0 || ov.cluster_size > 0 || ov.cluster_stages > 0 ||
+                      ov.cluster_threads > 0 || ov.cluster_ctas_per_sm > 0 ||
+                      ov.stream_chunk_bytes > 0 || ov.stream_slots > 0 || ov.stream_hold >= 0 ||
+                      ov.stream_split_first >= 0 || ov.stream_prefetch_bytes >= 0 ||
+                      ov.stream_ctas_per_sm > 0 || ov.stream_cluster > 0 ||
+                      ov.stall_first_wait_ns > 0;
+  return !forced && !unal && row_bytes < kShortRowBytes;
+}
+// Warps per row and vectors per lane that hold a row of n_vec vectors.
+inline void short_shape(long long n_vec, int* warps, int* nv) {
+  *warps = n_vec <= 512 ? 1 : (n_vec <= 1024 ? 2 : 4);
+  *nv = n_vec <= 256 ? 8 : (n_vec <= 1024 ? 16 : 10);
+}
+
 // The ring. One CTA per SM, measured on GB300 among 44-112 KB chunks and 0-3
 // kept chunks (bf16, fused): rows of 240 KB and more run best with three 74
 // KB slots, the ragged remainder as the first chunk and the last two chunks
