@@ -488,8 +488,8 @@ rl_status launch_stats(const FwdIn& f, rl_loss_stats* stats, rl_loss_partials* p
   ta.ws = WsPtrs::at(f.ws, WsLayout::make(f.c.R, f.n_traj, f.n_groups));
   long long blocks = (f.c.R + kStatThreads - 1) / kStatThreads;  // one row per thread
   blocks = std::max<long long>(1, std::min<long long>(blocks, kMaxStatBlocks));
-  return launch(stats_kernel(), dim3(static_cast<unsigned>(blocks)), dim3(kStatThreads), 0, 1, s,
-                &ta, pdl);
+  return launch(stats_kernel(), dim3(static_cast<unsigned>(blocks)), dim3(kStatThreads), 0,
+                blocks <= kStatCluster ? static_cast<int>(blocks) : 1, s, &ta, pdl);
 }
 
 // phase: RL_PHASE_BEGIN (advantages, N), RL_PHASE_ROWS (the sweep over rows
@@ -535,8 +535,8 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
   aa.advantages = f.out_adv;
   aa.group_sizes = f.out_gsize;
   aa.estimator = c.p->estimator;
-  // cu_seqlens, group ids, rewards
-  const size_t traj_bytes = (3 * static_cast<size_t>(f.n_traj) + 1) * sizeof(int);
+  // cu_seqlens, group ids, rewards, advantages
+  const size_t traj_bytes = (4 * static_cast<size_t>(f.n_traj) + 1) * sizeof(int);
   aa.smem_traj = traj_bytes <= static_cast<size_t>(kAdvSmemBytes);
   aa.ws = ws;
   aa.groups_done = group_kernel_pays(f.n_groups, f.n_traj);

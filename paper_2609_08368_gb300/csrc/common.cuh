@@ -47,6 +47,7 @@ struct StatPart {
 
 constexpr int kMaxTopK = 64;
 constexpr int kStatThreads = 256;
+constexpr int kStatCluster = 8;      // up to this many blocks run as one cluster
 constexpr int kMaxStatBlocks = 256;  // one partial per thread of the final block
 
 struct WsLayout {
@@ -304,6 +305,10 @@ __device__ __forceinline__ float4 ld_dsmem_f4(uint32_t addr) {
                : "r"(addr)
                : "memory");
   return v;
+}
+
+__device__ __forceinline__ void st_dsmem_f64(uint32_t addr, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
 }
 
 // Asynchronous 16-byte store into the shared memory of a CTA of the cluster

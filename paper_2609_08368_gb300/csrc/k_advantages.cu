@@ -42,19 +42,35 @@ __device__ __forceinline__ float warp_maxf(float v) {
   return v;
 }
 
-// Block-wide sum / maximum in a fixed order (valid in every thread): warp
-// butterflies, then every warp merges the warps' values by another (one
-// double operation per step and warp; a serial loop over the warps in every
-// thread queued 32 x 32 of them on the SM's double unit, 8 us a sum).
-template <bool kMax>
-__device__ double block_merge_d(double v, double* sh) {
+// Block-wide merges in a fixed order (valid in every thread): butterflies in
+// the warps that hold trajectories, then one over the warps' values, by warp
+// 0. A double operation holds the SM's double unit for 16 clocks a warp: when
+// every thread summed the warps' values by itself, 32 x 32 of them queued, 8 us
+// a merge.
+constexpr int kMergeMax = 3;
+template <int N>
+__device__ void block_merge_d(double (&v)[N], const bool (&is_max)[N], int n_traj,
+                              double (&sh)[kMergeMax][kWarps + 1]) {
+  static_assert(N <= kMergeMax, "merge scratch");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  v = kMax ? warp_max(v) : warp_sum(v);
   __syncthreads();
-  if (lane == 0) sh[warp] = v;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    if (warp * 32 < n_traj) v[i] = is_max[i] ? warp_max(v[i]) : warp_sum(v[i]);
+    if (lane == 0) sh[i][warp] = v[i];
+  }
   __syncthreads();
-  double t = lane < kWarps ? sh[lane] : (kMax ? -INFINITY : 0.0);
-  return kMax ? warp_max(t) : warp_sum(t);
+  if (warp == 0) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      double t = lane < kWarps ? sh[i][lane] : (is_max[i] ? -INFINITY : 0.0);
+      t = is_max[i] ? warp_max(t) : warp_sum(t);
+      if (lane == 0) sh[i][kWarps] = t;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] = sh[i][kWarps];
 }
 
 // The statistics of group g, computed by one warp that scans the group ids
@@ -127,16 +143,18 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
   const int gtid = rank * kAdvThreads + tid, gthreads = NC * kAdvThreads;
   const int gwarp = rank * kWarps + warp, gwarps = NC * kWarps;
   __shared__ unsigned int s_err;
-  __shared__ double s_red[kWarps];
+  __shared__ double s_red[kMergeMax][kWarps + 1];
   __shared__ unsigned long long s_tok;
   __shared__ unsigned int s_seq;
   WsPtrs ws = a.ws;
-  // Shared copies, when they fit, of cu (n_traj + 1), group ids and rewards.
+  // Shared copies, when they fit, of cu (n_traj + 1), group ids and rewards,
+  // and the advantages of this CTA's trajectories.
   const bool on_chip = a.smem_traj;
   const int nt = a.n_traj;
   const int* cu = on_chip ? dyn : a.cu;
   const int* gid = on_chip ? dyn + (nt + 1) : a.gid;
   const float* rew = on_chip ? reinterpret_cast<const float*>(dyn + (2 * nt + 1)) : a.rewards;
+  float* adv_s = reinterpret_cast<float*>(dyn + (3 * nt + 1));
   if (tid == 0) {
     s_err = 0;
     s_tok = 0;
@@ -172,9 +190,10 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
   if (tid == 0 && (cu[0] != 0 || static_cast<long long>(cu[nt]) != a.R_total)) err |= kErrSeqlens;
   if (err) atomicOr(&s_err, err);
 
-  // ---- group statistics, one warp per group
+  // ---- group statistics, one warp per group, the groups dealt to the CTAs in
+  // turn
   if (!a.groups_done)
-    for (int g = gwarp; g < a.n_groups; g += gwarps) group_stats(a, gid, rew, g, lane);
+    for (int g = warp * NC + rank; g < a.n_groups; g += gwarps) group_stats(a, gid, rew, g, lane);
   // every CTA's part of the header, the counts and the group table is written
   __syncthreads();
   cluster_sync_all();
@@ -256,6 +275,29 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
       }
     }
   };
+  // The advantages of the trajectories whose rows this CTA writes, one thread
+  // each (a warp's lanes share each double operation), before the row pass.
+  // A trajectory shared by several CTAs is published by its first.
+  auto own_adv = [&](auto value_of) {
+    if (on_chip) {
+      const int g0 = rank * kWarps / wpt, g1 = (rank * kWarps + kWarps - 1) / wpt;
+      for (int i = tid; i < nt; i += kAdvThreads) {
+        const int g = i % traj_groups;
+        if (g < g0 || g > g1) continue;
+        const float A = value_of(i);
+        adv_s[i] = A;
+        if (g * wpt >= rank * kWarps) publish(i, A);
+      }
+      __syncthreads();
+    }
+  };
+  auto adv_of = [&](int i, auto value_of) {
+    if (on_chip) return adv_s[i];
+    const float A = value_of(i);
+    if (sub == 0 && lane == 0) publish(i, A);
+    return A;
+  };
+  auto direct = [&](int i) { return static_cast<float>(base_value(i)); };
   unsigned long long n_tok = 0;  // (lane 0 of each warp, or every thread's own)
   unsigned int n_seq = 0;
   if (lookup) {
@@ -266,6 +308,7 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
         n_tok += static_cast<unsigned long long>(c);
         n_seq += c > 0;
       }
+    if (!rpp) own_adv(direct);
     if (group < traj_groups)
       for (int i = group; i < nt; i += traj_groups) {
         const long long lo = local_lo(i), hi = local_hi(i);
@@ -277,11 +320,7 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
             n_tok += static_cast<unsigned long long>(c);
           }
         }
-        if (!rpp) {
-          const float A = static_cast<float>(base_value(i));
-          if (sub == 0 && lane == 0) publish(i, A);
-          write_rows(lo, hi, A);
-        }
+        if (!rpp) write_rows(lo, hi, adv_of(i, direct));
       }
   } else {
     for (long long t = gtid; t < a.R; t += gthreads) {
@@ -318,9 +357,13 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
     bmax = fmax(bmax, b);
     bmin = fmin(bmin, b);
   }
-  sb = block_merge_d<false>(sb, s_red);
-  bmax = block_merge_d<true>(bmax, s_red);
-  bmin = -block_merge_d<true>(-bmin, s_red);
+  {
+    double v[3] = {sb, bmax, -bmin};
+    block_merge_d<3>(v, {false, true, true}, nt, s_red);
+    sb = v[0];
+    bmax = v[1];
+    bmin = -v[2];
+  }
   const bool zero_all = !(N > 0.0) || !(bmax != bmin);
   const double mu = N > 0.0 ? sb / N : 0.0;
   double ss = 0.0;
@@ -330,7 +373,11 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
     const double d = base_value(i) - mu;
     ss += d * d * n_i;
   }
-  ss = block_merge_d<false>(ss, s_red);
+  {
+    double v[1] = {ss};
+    block_merge_d<1>(v, {false}, nt, s_red);
+    ss = v[0];
+  }
   double den = 1.0;
   if (a.normalize_std) {
     const double ddof = a.unbiased_std ? 1.0 : 0.0;
@@ -340,12 +387,13 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
   auto final_value = [&](int i) {
     return static_cast<float>(zero_all ? 0.0 : (base_value(i) - mu) / den);
   };
-  for (int i = gtid; i < nt; i += gthreads) publish(i, final_value(i));
   if (lookup) {
+    own_adv(final_value);
     if (group < traj_groups)
       for (int i = group; i < nt; i += traj_groups)
-        write_rows(local_lo(i), local_hi(i), final_value(i));
+        write_rows(local_lo(i), local_hi(i), adv_of(i, final_value));
   } else {
+    for (int i = gtid; i < nt; i += gthreads) publish(i, final_value(i));
     for (long long t = gtid; t < a.R; t += gthreads) ws.a_row[t] = -opd(t);
   }
 }

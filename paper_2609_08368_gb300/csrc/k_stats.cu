@@ -4,9 +4,10 @@
 // correction ratio (Sec. 3.4), min / max ratio, and exact clip counts.
 //
 // Each block reduces a fixed strided set of rows into partial results
-// (butterfly merges in a fixed order), stores them in the workspace, and the
-// last block to finish (an atomic ticket, no waiting) merges the partials in
-// double precision in a fixed order. The grid size depends only on the row
+// (butterfly merges in a fixed order), which are merged in double precision in
+// a fixed order: of up to kStatCluster blocks through the shared memory of a
+// cluster, of more by the last block to finish (an atomic ticket, no waiting)
+// through the workspace. The grid size depends only on the row
 // count, so the scalar loss is bit-for-bit reproducible.
 //
 // Latency bounds the kernel (13 reads per row, 80 bytes, of rows the sweep has
@@ -25,7 +26,7 @@ namespace milesloss {
 namespace {
 
 // Per-block partial sums: fp32 within a block (a fixed-order tree over at
-// most kStatThreads rows; its rounding is far below the statistics'
+// most kStatThreads rows a block; its rounding is far below the statistics'
 // tolerance), exact integer counts.
 struct Part {
   float v[9];  // ell, pg, k3, H, r, |r-1|, |logp-rho|, rc, |rc-1|
@@ -84,6 +85,7 @@ static_assert(offsetof(rl_loss_stats, corr_absdev_mean) == 8 * sizeof(double) &&
 
 __global__ void __launch_bounds__(kStatThreads) k_stats(const StatArgs a) {
   constexpr int kWarps = kStatThreads / 32, kSubs = kStatThreads / kStatFields;
+  static_assert(kWarps >= kStatCluster, "one row of sh_d per warp, or per block of a cluster");
   __shared__ float sh_f[kWarps][kStatFields];         // the warps' sums and extremes
   __shared__ unsigned int sh_c[kWarps][kStatFields];  // ... and counts
   __shared__ double sh_d[kWarps][kStatFields];
@@ -145,7 +147,19 @@ __global__ void __launch_bounds__(kStatThreads) k_stats(const StatArgs a) {
       mine = static_cast<double>(v);
     }
   }
-  if (gridDim.x > 1) {
+  const int NC = static_cast<int>(cluster_nctarank());
+  if (gridDim.x > 1 && static_cast<int>(gridDim.x) == NC) {
+    // one cluster: every block's results into the first block's shared memory
+    const uint32_t rank = cluster_ctarank();
+    if (tid < kStatFields)
+      st_dsmem_f64(mapa_shared(smem_u32(&sh_d[rank][q]), 0), mine);
+    cluster_sync_all();
+    if (rank != 0) return;
+    if (tid < kStatFields) {
+      mine = sh_d[0][q];
+      for (int b = 1; b < NC; ++b) mine = merge_q(q, mine, sh_d[b][q]);
+    }
+  } else if (gridDim.x > 1) {
     if (warp == 0) {
       if (lane < kStatFields) {
         ws.parts[blockIdx.x].f[lane] = mine;

@@ -134,8 +134,8 @@ struct AdvArgs {
   int normalize_std, unbiased_std;
   float std_floor;
   int estimator;   // rl_estimator
-  int smem_traj;   // trajectory tables (cu_seqlens, group ids, rewards) staged in
-                   // shared memory
+  int smem_traj;   // trajectory tables (cu_seqlens, group ids, rewards, advantages)
+                   // staged in shared memory
   int groups_done; // k_groups has computed the group statistics
   float* advantages;   // may be null
   int* group_sizes;    // may be null
