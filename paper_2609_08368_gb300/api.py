@@ -444,24 +444,36 @@ def vocab_sharded_fwd_bwd_local(shards):
     GPU), ``shards[i][k]`` the column shard k of row shard i: the exchanges
     are sums, stacks and maxima over the shards' tensors."""
     flat = [s for row in shards for s in row]
+    # With one row shard there is nothing to add up over the row shards: its
+    # column shards hold the same counts, sums and partials already (a dozen
+    # small tensor operations fewer, each more host time than its kernel).
+    one = len(shards) == 1
     for s in flat:
         s.count()
-    total = torch.stack([row[0].counts for row in shards]).sum(0)
+    if not one:
+        total = torch.stack([row[0].counts for row in shards]).sum(0)
     for s in flat:
-        s.counts.copy_(total)
+        if not one:
+            s.counts.copy_(total)
         s.partial()
     for row in shards:
-        gathered = torch.stack([s.row_partials for s in row])
+        gathered = row[0].row_partials_all
+        torch.stack([s.row_partials for s in row], out=gathered)
         for s in row:
-            s.row_partials_all.copy_(gathered)
+            if s is not row[0]:
+                s.row_partials_all.copy_(gathered)
             s.sweep()
     if flat and flat[0].gspo:
-        sums = torch.stack([row[0].traj_sums for row in shards]).sum(0)
+        if not one:
+            sums = torch.stack([row[0].traj_sums for row in shards]).sum(0)
         for s in flat:
-            s.traj_sums.copy_(sums)
+            if not one:
+                s.traj_sums.copy_(sums)
             s.seq()
-    p = torch.stack([row[0].partials for row in shards])
-    comb = torch.cat([p[:, :ml.PARTIALS_SUMS].sum(0), p[:, ml.PARTIALS_SUMS:].max(0).values])
+    if not one:
+        p = torch.stack([row[0].partials for row in shards])
+        comb = torch.cat([p[:, :ml.PARTIALS_SUMS].sum(0), p[:, ml.PARTIALS_SUMS:].max(0).values])
     for s in flat:
-        s.partials.copy_(comb)
+        if not one:
+            s.partials.copy_(comb)
         s.finish()

@@ -419,10 +419,8 @@ void record(cudaEvent_t ev, cudaStream_t s) {
 // The gradient sweep from the per-row state in the workspace (lse, H, G).
 rl_status launch_bwd(const Common& c, const GradOut& go, const WsPtrs& ws, cudaStream_t s,
                      long long col0, bool pdl) {
-  int dev = 0, sms = 0;
+  int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return RL_ERR_CUDA;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return RL_ERR_CUDA;
   BwdArgs b;
   b.logits = c.logits;
   b.ld = c.ld;
@@ -446,11 +444,10 @@ rl_status launch_bwd(const Common& c, const GradOut& go, const WsPtrs& ws, cudaS
   // one wave of resident blocks (grid-stride over the tiles): a second,
   // partial wave would run with fewer loads in flight
   const void* fn = bwd_kernel(c.dt, go.dt, unal);
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBwdThreads, 0) != cudaSuccess)
-    return RL_ERR_CUDA;
-  const long long grid =
-      std::min<long long>(b.n_tiles, static_cast<long long>(sms) * std::max(per_sm, 1));
+  int resident = 0;
+  const rl_status st = resident_clusters(fn, dev, 1, 0, kBwdThreads, &resident);
+  if (st != RL_OK) return st;
+  const long long grid = std::min<long long>(b.n_tiles, resident);
   return launch(fn, dim3(static_cast<unsigned>(grid)), dim3(kBwdThreads), 0, 1, s, &b,
                 pdl);
 }
@@ -539,14 +536,19 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
   const size_t traj_bytes = (4 * static_cast<size_t>(f.n_traj) + 1) * sizeof(int);
   aa.smem_traj = traj_bytes <= static_cast<size_t>(kAdvSmemBytes);
   aa.ws = ws;
+  // Small calls, where launches count, start while whatever ran before them
+  // ends (eager calls of 2,048 x 4,096 23.1 -> 20 us); past that the waiting
+  // CTAs are in the way as often as they help (3,488 x 43,648 with top-K 127.0
+  // -> 132.0 us, two vocabulary shards of 4,096 rows 657 -> 645).
+  const bool early = overlap && c.R <= kEarlyStartRows;
   aa.groups_done = group_kernel_pays(f.n_groups, f.n_traj);
   if (aa.groups_done) {
     const int gb = std::min(f.n_groups, kMaxGroupBlocks);
-    st = launch(groups_kernel(), dim3(static_cast<unsigned>(gb)), dim3(32), 0, 1, s, &aa);
+    st = launch(groups_kernel(), dim3(static_cast<unsigned>(gb)), dim3(32), 0, 1, s, &aa, early);
     if (st != RL_OK) return st;
   }
   st = launch(adv_kernel(), dim3(kAdvCluster), dim3(kAdvThreads),
-              aa.smem_traj ? static_cast<int>(traj_bytes) : 0, kAdvCluster, s, &aa);
+              aa.smem_traj ? static_cast<int>(traj_bytes) : 0, kAdvCluster, s, &aa, early);
   if (st != RL_OK) return st;
   pdl = overlap;
   }

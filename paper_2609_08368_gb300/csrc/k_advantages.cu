@@ -131,13 +131,18 @@ __device__ void group_stats(const AdvArgs& a, const int* gid, const float* rew, 
 // Group statistics for calls whose groups are too many for one cluster
 // (group_kernel_pays), one 32-thread block per group over the whole GPU.
 __global__ void __launch_bounds__(32) k_groups(const AdvArgs a) {
+  pdl_wait();
+  pdl_trigger();
   for (int g = blockIdx.x; g < a.n_groups; g += gridDim.x)
     group_stats(a, a.gid, a.rewards, g, threadIdx.x);
 }
 
 __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) {
   extern __shared__ __align__(16) int dyn[];
-  pdl_trigger();  // (launched as an ordinary kernel: whatever ran before it has finished)
+  // whatever ran before the call has finished once this returns; only then may
+  // the sweep start, which reads the call's inputs without waiting for them
+  pdl_wait();
+  pdl_trigger();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = static_cast<int>(cluster_ctarank()), NC = static_cast<int>(cluster_nctarank());
   const int gtid = rank * kAdvThreads + tid, gthreads = NC * kAdvThreads;

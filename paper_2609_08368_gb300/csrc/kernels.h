@@ -11,6 +11,7 @@ namespace milesloss {
 constexpr int kMaxStages = 4;
 constexpr int kMaxCluster = 8;
 constexpr uint32_t kBulkChunk = 16384;    // bytes per cp.async.bulk
+constexpr int kEarlyStartRows = 2048;     // calls of up to this many rows overlap what ran before
 constexpr int kAdvThreads = 512;
 // CTAs of the advantage kernel (one cluster). With 1 / 4 / 8: 512 trajectories of
 // 64 rows x 32,768 fp32 1,426 / 1,337 / 1,327 us a call, 128 x 128 rows x 20,480

