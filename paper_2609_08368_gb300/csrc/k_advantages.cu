@@ -77,8 +77,13 @@ __device__ void block_merge_d(double (&v)[N], const bool (&is_max)[N], int n_tra
 // for the group's members: n, mean, the standard deviation with its floor,
 // and whether all rewards are equal. In double precision; a step of the scan
 // that meets no member adds nothing and skips the double arithmetic.
-__device__ void group_stats(const AdvArgs& a, const int* gid, const float* rew, int g, int lane) {
-  WsPtrs ws = a.ws;
+struct Group {
+  int n, flat;
+  double mu, den;
+};
+__device__ __forceinline__ Group group_stats(const AdvArgs& a, const int* gid, const float* rew,
+                                             int g, int lane) {
+  Group r;
   int n = 0;
   double sum = 0.0;
   float wmax = -INFINITY, wmin = INFINITY;
@@ -95,16 +100,16 @@ __device__ void group_stats(const AdvArgs& a, const int* gid, const float* rew, 
       wmin = fminf(wmin, w);
     }
   }
-  n = __reduce_add_sync(0xffffffffu, n);
+  r.n = n = __reduce_add_sync(0xffffffffu, n);
   sum = warp_sum(sum);
   wmax = warp_maxf(wmax);
   wmin = -warp_maxf(-wmin);
-  const double mu = n > 0 ? sum / n : 0.0;
+  r.mu = n > 0 ? sum / n : 0.0;
   // A group whose rewards are all equal (this includes one-member groups)
   // carries no advantage signal: its GRPO advantages are exactly zero.
-  const int flat = (n == 0) || (wmax == wmin);
-  double den = 1.0;
-  if (a.normalize_std && !flat) {  // (uniform over the warp)
+  r.flat = (n == 0) || (wmax == wmin);
+  r.den = 1.0;
+  if (a.normalize_std && !r.flat) {  // (uniform over the warp)
     double ss = 0.0;
 #pragma unroll 4
     for (int b = 0; b < a.n_traj; b += 32) {
@@ -112,20 +117,21 @@ __device__ void group_stats(const AdvArgs& a, const int* gid, const float* rew, 
       const bool in = i < a.n_traj && gid[i] == g;
       if (!__any_sync(0xffffffffu, in)) continue;
       if (in) {
-        const double d = static_cast<double>(rew[i]) - mu;
+        const double d = static_cast<double>(rew[i]) - r.mu;
         ss += d * d;
       }
     }
     ss = warp_sum(ss);
     const int ddof = a.unbiased_std ? 1 : 0;
-    den = fmax(sqrt(ss / static_cast<double>(n - ddof)), static_cast<double>(a.std_floor));
+    r.den = fmax(sqrt(ss / static_cast<double>(n - ddof)), static_cast<double>(a.std_floor));
   }
-  if (lane == 0) {
-    ws.g_mu[g] = mu;
-    ws.g_den[g] = den;
-    ws.g_flag[g] = flat;
-    if (a.group_sizes) a.group_sizes[g] = n;
-  }
+  return r;
+}
+__device__ __forceinline__ void group_store(const AdvArgs& a, const Group& r, int g) {
+  a.ws.g_mu[g] = r.mu;
+  a.ws.g_den[g] = r.den;
+  a.ws.g_flag[g] = r.flat;
+  if (a.group_sizes) a.group_sizes[g] = r.n;
 }
 
 // Group statistics for calls whose groups are too many for one cluster
@@ -133,8 +139,10 @@ __device__ void group_stats(const AdvArgs& a, const int* gid, const float* rew, 
 __global__ void __launch_bounds__(32) k_groups(const AdvArgs a) {
   pdl_wait();
   pdl_trigger();
-  for (int g = blockIdx.x; g < a.n_groups; g += gridDim.x)
-    group_stats(a, a.gid, a.rewards, g, threadIdx.x);
+  for (int g = blockIdx.x; g < a.n_groups; g += gridDim.x) {
+    const Group r = group_stats(a, a.gid, a.rewards, g, threadIdx.x);
+    if (threadIdx.x == 0) group_store(a, r, g);
+  }
 }
 
 __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) {
@@ -198,7 +206,10 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
   // ---- group statistics, one warp per group, the groups dealt to the CTAs in
   // turn
   if (!a.groups_done)
-    for (int g = warp * NC + rank; g < a.n_groups; g += gwarps) group_stats(a, gid, rew, g, lane);
+    for (int g = warp * NC + rank; g < a.n_groups; g += gwarps) {
+      const Group r = group_stats(a, gid, rew, g, lane);
+      if (lane == 0) group_store(a, r, g);
+    }
   // every CTA's part of the header, the counts and the group table is written
   __syncthreads();
   cluster_sync_all();
@@ -403,8 +414,157 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
   }
 }
 
+// The usual call: GRPO, with the trajectory tables on chip and no counts asked
+// for (k_advantages does the rest). No CTA waits for another: the last counts
+// N, checks the inputs and writes the header and the group sizes; every other
+// one has a run of trajectories (or, with few trajectories, a piece of one),
+// forms the statistics of the groups they belong to (each by one warp, in
+// k_advantages' order: the same bits), and writes their advantages and rows.
+// What bounds it is one chain: tables, a group's double arithmetic, the rows;
+// it ends before the sweep's first row needs it. k_advantages, with two
+// barriers of the cluster and the group table's way through L2 in the chain,
+// took 7.3-8.3 us from its start on 2,048 rows: with this kernel an eager call of
+// 2,048 x 4,096 went from 19.1 to 16.6 us, 3,136 x 15,616 (224 trajectories) 56.2 ->
+// 49.8, 27,456 x 33,247 710 -> 682, 32,768 x 32,768 fp32 1,307 -> 1,290.
+__global__ void __launch_bounds__(kAdvThreads, 1) k_adv_grpo(const AdvArgs a) {
+  extern __shared__ __align__(16) int dyn[];
+  pdl_wait();  // as in k_advantages
+  pdl_trigger();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nt = a.n_traj;
+  __shared__ unsigned int s_err;
+  __shared__ unsigned int s_cnt[kWarps];
+  int* cu = dyn;
+  int* gid = dyn + (nt + 1);
+  float* rew = reinterpret_cast<float*>(dyn + (2 * nt + 1));
+  float* adv_s = reinterpret_cast<float*>(dyn + (3 * nt + 1));
+  WsPtrs ws = a.ws;
+  if (tid == 0) s_err = 0;
+  for (int i = tid; i <= nt; i += kAdvThreads) {
+    cu[i] = a.cu[i];
+    if (i < nt) {
+      gid[i] = a.gid[i];
+      rew[i] = a.rewards[i];
+    }
+  }
+  const int n_row_ctas = static_cast<int>(gridDim.x) - 1;
+  const bool counts = static_cast<int>(blockIdx.x) == n_row_ctas;
+  unsigned int n_tok = 0;
+  if (counts && !a.counts_in) {
+    const long long whole = (reinterpret_cast<uintptr_t>(a.mask) & 15u) == 0 ? a.R / 16 : 0;
+#pragma unroll 4
+    for (long long b = tid; b < whole; b += kAdvThreads) {
+      const uint4 v = reinterpret_cast<const uint4*>(a.mask)[b];
+      n_tok += (__popc(__vcmpne4(v.x, 0u)) + __popc(__vcmpne4(v.y, 0u)) +
+                __popc(__vcmpne4(v.z, 0u)) + __popc(__vcmpne4(v.w, 0u))) >> 3;
+    }
+    for (long long t = whole * 16 + tid; t < a.R; t += kAdvThreads) n_tok += a.mask[t] != 0;
+  }
+  __syncthreads();
+  unsigned int err = 0;
+  for (int i = tid; i < nt; i += kAdvThreads) {
+    if (cu[i] > cu[i + 1]) err |= kErrSeqlens;
+    const int g = gid[i];
+    if (g < 0 || g >= a.n_groups) err |= kErrGroup;
+    if (counts && a.counts_in) n_tok += static_cast<unsigned int>(a.counts_in[i]);
+  }
+  if (tid == 0 && (cu[0] != 0 || static_cast<long long>(cu[nt]) != a.R_total)) err |= kErrSeqlens;
+  if (err) atomicOr(&s_err, err);
+  n_tok = __reduce_add_sync(0xffffffffu, n_tok);
+  if (lane == 0) s_cnt[warp] = n_tok;
+
+  if (counts) {
+    __syncthreads();
+    if (tid == 0) {
+      long long N = 0;
+      for (int w = 0; w < kWarps; ++w) N += s_cnt[w];
+      ws.hdr->err_bits = s_err;
+      ws.hdr->ticket = 0;
+      ws.hdr->n_tokens = N;
+      ws.hdr->n_seq = 0;  // (GSPO's)
+    }
+    if (a.group_sizes)
+      for (int g = warp; g < a.n_groups; g += kWarps) {
+        int n = 0;
+        for (int i = lane; i < nt; i += 32) n += gid[i] == g;
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (lane == 0) a.group_sizes[g] = n;
+      }
+    return;
+  }
+
+  // This CTA's trajectories [i0, i1) and, with more CTAs than trajectories,
+  // which of `pieces` pieces of its one trajectory's rows.
+  const int pieces = max(1, n_row_ctas / nt);
+  const int b = static_cast<int>(blockIdx.x);
+  const int per = (nt + n_row_ctas - 1) / n_row_ctas;
+  const int i0 = min(nt, pieces > 1 ? b / pieces : b * per);
+  const int i1 = min(nt, pieces > 1 ? i0 + 1 : i0 + per);
+  const int piece = pieces > 1 ? b % pieces : 0;
+  for (int i = i0 + warp; i < i1; i += kWarps) {
+    // the first of the run's members of a group does the group
+    const int g = gid[i];
+    bool later = false;
+    for (int m = i0 + lane; m < i; m += 32) later |= gid[m] == g;
+    if (__any_sync(0xffffffffu, later)) continue;
+    Group r{0, 1, 0.0, 1.0};
+    if (g >= 0 && g < a.n_groups) r = group_stats(a, gid, rew, g, lane);
+    for (int m = i0 + lane; m < i1; m += 32) {
+      if (gid[m] != g) continue;
+      const float A =
+          r.flat ? 0.0f : static_cast<float>((static_cast<double>(rew[m]) - r.mu) / r.den);
+      adv_s[m] = A;
+      if (piece == 0) {
+        ws.a_traj[m] = A;
+        if (a.advantages) a.advantages[m] = A;
+      }
+    }
+  }
+  __syncthreads();
+  const bool cu_ok = (s_err & kErrSeqlens) == 0;
+  auto opd = [&](long long t) { return a.teacher ? a.opd_coef * (a.rho[t] - a.teacher[t]) : 0.0f; };
+  if (!cu_ok) {  // rows cannot be attributed: advantage 0 (plus the shaping)
+    for (long long t = static_cast<long long>(b) * kAdvThreads + tid; t < a.R;
+         t += static_cast<long long>(n_row_ctas) * kAdvThreads)
+      ws.a_row[t] = -opd(t);
+    return;
+  }
+  // the rows of the run, four to a thread, a warp (or a piece's warps) per trajectory
+  const int wpt = max(1, kWarps / max(1, i1 - i0));
+  const int n_par = max(1, kWarps / wpt);
+  const bool vec = ((reinterpret_cast<uintptr_t>(ws.a_row) |
+                     (a.teacher ? reinterpret_cast<uintptr_t>(a.rho) |
+                                      reinterpret_cast<uintptr_t>(a.teacher)
+                                : 0u)) & 15u) == 0;
+  if (warp / wpt >= n_par) return;
+  for (int i = i0 + warp / wpt; i < i1; i += n_par) {
+    const long long lo = max(static_cast<long long>(cu[i]), a.row0) - a.row0;
+    const long long hi = max(min(static_cast<long long>(cu[i + 1]), a.row0 + a.R) - a.row0, lo);
+    const float A = adv_s[i];
+    const long long step = 4LL * 32 * wpt * pieces;
+    for (long long t0 = (lo & ~3LL) + 4LL * (lane + 32 * (warp % wpt + wpt * piece)); t0 < hi;
+         t0 += step) {
+      if (vec && t0 >= lo && t0 + 4 <= hi) {
+        float4 v = make_float4(A, A, A, A);
+        if (a.teacher) {
+          const float4 p = *reinterpret_cast<const float4*>(a.rho + t0);
+          const float4 q = *reinterpret_cast<const float4*>(a.teacher + t0);
+          v.x -= a.opd_coef * (p.x - q.x);
+          v.y -= a.opd_coef * (p.y - q.y);
+          v.z -= a.opd_coef * (p.z - q.z);
+          v.w -= a.opd_coef * (p.w - q.w);
+        }
+        *reinterpret_cast<float4*>(ws.a_row + t0) = v;
+      } else {
+        for (long long t = max(t0, lo); t < min(t0 + 4, hi); ++t) ws.a_row[t] = A - opd(t);
+      }
+    }
+  }
+}
+
 }  // namespace
 
+const void* adv_grpo_kernel() { return reinterpret_cast<const void*>(&k_adv_grpo); }
 const void* adv_kernel() { return reinterpret_cast<const void*>(&k_advantages); }
 const void* groups_kernel() { return reinterpret_cast<const void*>(&k_groups); }
 

@@ -250,6 +250,15 @@ rl_status plan_stream(int dev, int extra, long long row_bytes, int es, bool grad
                       bool unal, bool can_cluster, const rl_launch_overrides& ov, StreamPlan* out);
 const void* bwd_kernel(rl_dtype in, rl_dtype out, bool unal);
 const void* adv_kernel();
+const void* adv_grpo_kernel();  // GRPO without counts: a grid of adv_grpo_ctas
+// CTAs of k_adv_grpo: one that counts, and one per four groups' worth of
+// trajectories (a group's double arithmetic is some 0.3 us of its SM) or per
+// 2,048 rows.
+inline int adv_grpo_ctas(long long rows, int n_traj) {
+  const long long by_rows = (rows + 2047) / 2048, by_traj = (n_traj + 15) / 16;
+  const long long n = by_rows > by_traj ? by_rows : by_traj;
+  return static_cast<int>(n < 1 ? 1 : (n > 32 ? 32 : n)) + 1;
+}
 const void* groups_kernel();  // one 32-thread block per group (grid-stride)
 constexpr int kMaxGroupBlocks = 65535;
 // k_advantages computes the group statistics itself unless its cluster's
