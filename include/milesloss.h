@@ -193,11 +193,10 @@ rl_status rl_loss_workspace_size(int64_t n_rows, int32_t n_traj, int32_t n_group
  *                    by the caller); only the first `vocab` columns are read.
  *                    Rows whose start is 16-byte aligned (ld * element size a
  *                    multiple of 16 and a 16-byte aligned base) are fastest;
- *                    any other layout is correct (bf16 rows are then copied
- *                    in the 16-byte granules they touch, so the neighbours'
- *                    bytes in a row's first and last granule are fetched too,
- *                    never bytes outside the rows; fp32 rows go element by
- *                    element).
+ *                    any other layout is correct (rows are then copied in the
+ *                    16-byte granules they touch, so the neighbours' bytes in
+ *                    a row's first and last granule are fetched too, never
+ *                    bytes outside the rows).
  *  targets           [n_rows] int32 sampled token ids, in [0, vocab)
  *  rollout_logprobs  [n_rows] fp32 log-probs the rollout engine reported
  *  ref_logprobs      [n_rows] fp32 reference-policy log-probs, or NULL

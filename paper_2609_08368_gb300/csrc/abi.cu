@@ -595,11 +595,18 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
   // (unaligned rows whose ring, forced by an override, has no room for the
   // slots' padding: the cluster kernel)
   StreamPlan sp;
+  const bool virt = es == 4 && !in_bulk;  // summed in the cluster kernel's order
+  const int extra = (sc.topk ? kTopKSmem : 0) + (virt ? kVirtSmem : 0);
+  rl_launch_overrides pov = ov;
   bool stream = c.R > 0 && use_stream(row_bytes, static_cast<int>(es), in_bulk, unal, grad,
                                       sc.topk > 0, ov);
+  if (stream && virt) {
+    pov.stream_ctas_per_sm = 2;
+    pov.stream_cluster = 1;
+  }
   if (stream && unal) {
-    st = plan_stream(dev, sc.topk ? kTopKSmem : 0, row_bytes, static_cast<int>(es), grad,
-                     sc.topk > 0, unal, f.part_rows == nullptr, ov, &sp);
+    st = plan_stream(dev, extra, row_bytes, static_cast<int>(es), grad, sc.topk > 0, unal,
+                     f.part_rows == nullptr, pov, &sp);
     if (st == RL_ERR_UNSUPPORTED) stream = false;
     else if (st != RL_OK) return st;
   }
@@ -642,10 +649,14 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     const void* fn = nullptr;
     int ctas = 0;  // resident CTAs, or clusters of sp.cluster CTAs
     int threads = 0;
-    rl_launch_overrides pov = ov;
+    SweepPlan slices{};
+    if (virt) {
+      st = plan_sweep(c.dt, c.V, dev, sc.topk ? kTopKSmem : 0, grad, ov, &slices);
+      if (st != RL_OK) return st;
+    }
     for (;;) {
-      st = plan_stream(dev, sc.topk ? kTopKSmem : 0, row_bytes, static_cast<int>(es), grad,
-                       sc.topk > 0, unal, f.part_rows == nullptr, pov, &sp);
+      st = plan_stream(dev, extra, row_bytes, static_cast<int>(es), grad, sc.topk > 0, unal,
+                       f.part_rows == nullptr, pov, &sp);
       if (st != RL_OK) return st;
       fn = stream_kernel(c.dt, grad ? go->dt : c.dt, grad, sc.topk > 0, unal, sp.cw, sp.cluster > 1);
       if (!fn) return RL_ERR_UNSUPPORTED;
@@ -673,6 +684,8 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     ta.split_first = sp.split_first;
     ta.prefetch = sp.prefetch;
     ta.slice_vec = sp.slice_vec;
+    ta.virt_slice = virt ? slices.slice : 0;
+    ta.virt_c = virt ? slices.C : 1;
     ta.targets = c.targets;
     ta.rho = fr.rho;
     ta.q = fr.q;

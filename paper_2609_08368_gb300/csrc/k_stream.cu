@@ -8,10 +8,9 @@ namespace milesloss {
 bool use_stream(long long row_bytes, int es, bool in_bulk, bool unal, bool grad, bool topk,
                 const rl_launch_overrides& ov) {
   if (ov.sweep_kernel == 0) return false;
-  // Unaligned fp32 logits stay with the cluster kernel: their log-probs carry
-  // the order of its sums in the last bit, and the gradient of a token whose
-  // log-prob is near the reference's turns that into 2e-4 of an entry.
-  if (es == 4 && !in_bulk) return false;
+  // (unaligned fp32 logits: in the cluster kernel's order, k_stream.cuh; with
+  // a launch shape forced, and below kVirtRowBytes, by that kernel itself)
+  if (es == 4 && !in_bulk) return !plan_forced(ov) && row_bytes >= kVirtRowBytes;
   if (ov.sweep_kernel == 1) return true;
   return stream_ctas(row_bytes, es, grad, topk, unal && es == 2) > 0;
 }

@@ -44,6 +44,15 @@
 // granules of dLogits instead, with the few elements that share one with a
 // neighbouring row stored one by one. Before, such rows were read and written
 // element by element: 4,096 x 45,003 bf16 937 -> 135 us.
+// Unaligned fp32 rows keep the sums of the cluster kernel, which reads them
+// element by element: 256 threads per slice of the row, thread v the elements
+// v, v + 256, ... of it against a running maximum, the slices' sums merged in
+// order. Eight consumer warps stand in for one slice's threads after the
+// other's (virt_slice), from the slots. (A log-prob's last bit, where a token's
+// gradient is the difference to its reference's, is 2e-4 of a dLogit.)
+// Fused calls, against that kernel: 4,096 rows x 5,001 / 10,001 / 32,769 147 /
+// 237 / 667 -> 82 / 133 / 373 us, 2,048 x 130,003 2,085 -> 581, 1,024 x 230,003
+// 5,447 -> 567; the chain of a running maximum bounds it.
 // Definitions: Sec. 3.4 (ratio), Sec. 2 / 9.1 (advantage), Sec. 2.4 (mask).
 #pragma once
 
@@ -309,6 +318,12 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
                         6 * 8 + 2 * 8 + 8 + 2 * kMaxCluster * 16 <=
                     kSweepSmemExtra,
                 "k_stream scratch");
+  // (kUnal, fp32) the row's virtual slices (launched with kVirtSmem more): the
+  // sums of each slice's eight warps
+  constexpr bool kVirt = kUnal && V8 == 4 && kCW == 8 && !kClu;
+  const bool virt = kVirt && a.virt_slice > 0;
+  float4* vred = reinterpret_cast<float4*>(smem + static_cast<size_t>(NS) * CS + kSweepSmemExtra +
+                                           (kTopK ? kTopKSmem : 0));
   // [2] top-K candidates of this row and the next (launched with kTopKSmem more)
   TopKBuf* tkb = reinterpret_cast<TopKBuf*>(smem + static_cast<size_t>(NS) * CS + kSweepSmemExtra);
 
@@ -575,7 +590,12 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
     const int sh = shift_of(grow);
     // (kUnal) the thread's element past the last whole vector, loaded early
     float z_tail = 0.0f;
-    if (kUnal && my_tail0 + tid < a.V) z_tail = In::load1(grow, my_tail0 + tid);
+    int j_tail = my_tail0 + tid;
+    if (virt) {  // the one of its slice's thread
+      const int v = tid - ((tail0 - (a.virt_c - 1) * a.virt_slice) & 255);
+      j_tail = tail0 + (v & 255);
+    }
+    if (kUnal && j_tail < a.V) z_tail = In::load1(grow, j_tail);
 
     int y = 0;
     float rho = 0.0f, q = 0.0f, old = 0.0f, A = 0.0f, zy = 0.0f;
@@ -607,7 +627,52 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
     // -inf logit (NaN) redoes the chunk against the chunk's own maximum,
     // skipping -inf logits exactly.
     Run run;
-    for (int c = 0; c < n_chunks; ++c) {
+    Tri t{-INFINITY, 0.0f, 0.0f};
+    // (kVirt, and the elements past the last whole vector)
+    auto add1 = [&](float z) {
+      if (z == -INFINITY) return;
+      const float zk = z * k;
+      if (zk > t.m) {
+        if (t.s > 0.0f) {
+          const float d = t.m - zk, f = ex2(d);
+          t.u = f * fmaf(d, t.s, t.u);
+          t.s *= f;
+        }
+        t.m = zk;
+      }
+      const float tt = fmaf(z, k, -t.m), x = ex2(tt);
+      t.s += x;
+      t.u = fmaf(x, tt, t.u);
+    };
+    if constexpr (kVirt) {
+      if (virt) {
+        int vc = 0;
+        for (int c = 0; c < n_chunks; ++c) {
+          wait_slot(q0 + c);
+          const uint4* sv = slot(q0 + c);
+          const int v0 = cs(c), nv = cn(c);
+          if (tid == 0 && yv >= v0 && yv < v0 + nv) zy = In::load1(sv, y - v0 * V8 + sh);
+          const float* src = reinterpret_cast<const float*>(sv) + sh - v0 * V8;
+          const int e1 = (v0 + nv) * V8;
+          for (int e0 = v0 * V8; e0 < e1;) {
+            const int lo = vc * a.virt_slice;
+            const int end = vc == a.virt_c - 1 ? e1 : min(e1, lo + a.virt_slice);
+#pragma unroll 4
+            for (int j = e0 + ((tid - (e0 - lo)) & 255); j < end; j += 256) add1(src[j]);
+            e0 = end;
+            if (vc < a.virt_c - 1 && end == lo + a.virt_slice) {  // the slice is complete
+              t = warp_merge(t);
+              if (lane == 0) vred[vc * 8 + warp] = make_float4(t.m, t.s, t.u, 0.0f);
+              t = Tri{-INFINITY, 0.0f, 0.0f};
+              ++vc;
+            }
+          }
+          if (c < n_chunks - h) release_slot(q0 + c);
+        }
+        if (j_tail < a.V) add1(z_tail);
+      }
+    }
+    for (int c = virt ? n_chunks : 0; c < n_chunks; ++c) {
       wait_slot(q0 + c);
       const uint4* sv = slot(q0 + c);
       const int v0 = cs(c), nv = cn(c);
@@ -663,22 +728,10 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
       }
       if (c < n_chunks - h) release_slot(q0 + c);
     }
-    Tri t = run.tri();
-    for (int j = my_tail0 + tid; j < a.V; j += kCons) {
-      const float z = kUnal ? z_tail : In::load1(grow, j);  // (kUnal: at most one per thread)
-      if (z == -INFINITY) continue;
-      const float zk = z * k;
-      if (zk > t.m) {
-        if (t.s > 0.0f) {
-          const float d = t.m - zk, f = ex2(d);
-          t.u = f * fmaf(d, t.s, t.u);
-          t.s *= f;
-        }
-        t.m = zk;
-      }
-      const float tt = fmaf(z, k, -t.m), x = ex2(tt);
-      t.s += x;
-      t.u = fmaf(x, tt, t.u);
+    if (!virt) {
+      t = run.tri();
+      for (int j = my_tail0 + tid; j < a.V; j += kCons)
+        add1(kUnal ? z_tail : In::load1(grow, j));  // (kUnal: at most one per thread)
     }
 
     if (i == 0 && tid == 0) {
@@ -694,13 +747,46 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
     // ---------------- merge
     t = warp_merge(t);
     if (lane == 0) {
+      if (virt) vred[(a.virt_c - 1) * 8 + warp] = make_float4(t.m, t.s, t.u, 0.0f);
       red[warp] = make_float4(t.m, t.s, t.u, 0.0f);
       redm[warp] = t.m;
     }
     cons_sync<kCW>();
     if (tid == 0 && fix_ptr) Out::store1(fix_ptr, 0, fix_val);  // previous row's y entry
     fix_ptr = nullptr;
-    if (warp == 0) t = block_merge<kCW>(red, redm, lane);
+    if (virt) {
+      if constexpr (kVirt) {
+        if (warp == 0) {
+          // every slice's warps, then (thread 0) the slices in order
+          for (int c = 0; c < a.virt_c; ++c) {
+            t = Tri{-INFINITY, 0.0f, 0.0f};
+            if (lane < 8) {
+              const float4 v = vred[c * 8 + lane];
+              t = Tri{v.x, v.y, v.z};
+            }
+            t = warp_merge(t);
+            if (lane == 0) vred[c * 8] = make_float4(t.m, t.s, t.u, 0.0f);
+            __syncwarp();
+          }
+          if (a.virt_c > 1) {
+            float M = -INFINITY;
+            for (int c = 0; c < a.virt_c; ++c) M = fmaxf(M, vred[c * 8].x);
+            Tri tot{M, 0.0f, 0.0f};
+            for (int c = 0; c < a.virt_c; ++c) {
+              const float4 e = vred[c * 8];
+              if (e.y > 0.0f) {
+                const float d = e.x - M, f = ex2(d);
+                tot.s += f * e.y;
+                tot.u += f * fmaf(d, e.y, e.z);
+              }
+            }
+            t = tot;
+          }
+        }
+      }
+    } else if (warp == 0) {
+      t = block_merge<kCW>(red, redm, lane);
+    }
     bool cl_bad = false;  // (kClu, thread 0) a CTA of the cluster gave up before this row
     if constexpr (kClu) {
       if (tid == 0) {
@@ -909,8 +995,12 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
         edges([&](int e) { return value(In::load1(sv, sh + e)); });
         release_slot(qq);
       }
-      for (int j = my_tail0 + tid; j < a.V; j += kCons)
-        Out::store1(drow, j, value(kUnal ? z_tail : In::load1(grow, j)));
+      if constexpr (kUnal) {
+        if (j_tail < a.V) Out::store1(drow, j_tail, value(z_tail));
+      } else {
+        for (int j = my_tail0 + tid; j < a.V; j += kCons)
+          Out::store1(drow, j, value(In::load1(grow, j)));
+      }
     }
     q0 += (kGrad && trains) ? 2 * n_chunks - h : n_chunks;
   }

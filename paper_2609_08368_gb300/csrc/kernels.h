@@ -26,6 +26,7 @@ constexpr int stream_threads(bool topk, int cw) { return cw * 32 + (topk ? 64 : 
 constexpr int kShortThreads = 128;
 constexpr int kSeqThreads = 256;
 constexpr int kAdvSmemBytes = 48 * 1024;  // on-chip trajectory tables when they fit
+constexpr int kVirtSmem = kMaxCluster * 8 * 16;     // the warps' sums of a row's virtual slices
 constexpr int kTopKSmem = 2 * (2 * kMaxTopK * 4);  // two rows of top-K ids + teacher values
 
 struct SweepArgs {
@@ -73,6 +74,8 @@ struct StreamArgs {
   int n_hold;       // last chunks of a row that pass B reads from shared memory (<= n_slots)
   int split_first;  // 1: the first chunk takes the ragged remainder (rounded up to 128 bytes)
   int prefetch;     // bytes of the next row to ask L2 for once a row's first pass is issued
+  int virt_slice;   // > 0: unaligned fp32 rows, summed as virt_c slices of this many
+  int virt_c;       // elements are by the cluster kernel (k_stream.cuh)
   int slice_vec;    // launched in clusters (one per row): whole vectors of a row per CTA, a
                     // multiple of 8 (the cluster's last CTA may take fewer, or none)
   const int* targets;

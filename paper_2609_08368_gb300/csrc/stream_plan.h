@@ -61,8 +61,8 @@ inline bool halves_row(long long row_bytes, int es, bool grad, bool unal) {
   return grad && (es == 4 || unal) && row_bytes >= 136 * KB && row_bytes < 192 * KB;
 }
 
-// unal: rows that do not all start on a 16-byte boundary. The cluster kernel
-// reads and writes those element by element (4,096 x 45,003 bf16: 937 us
+// unal: bf16 rows that do not all start on a 16-byte boundary. The cluster
+// kernel reads and writes those element by element (4,096 x 45,003: 937 us
 // against 135), so every length streams: those the table above gives to the
 // cluster kernel with the CTAs per SM that came closest to it there.
 inline int stream_ctas(long long row_bytes, int es, bool grad, bool topk, bool unal = false) {
@@ -91,15 +91,20 @@ inline int stream_ctas(long long row_bytes, int es, bool grad, bool topk, bool u
 // dLogits): k_short, with the row in registers, unless an override asks for a
 // launch shape of the other kernels.
 constexpr long long kShortRowBytes = 20 * 1024;
-inline bool use_short(long long row_bytes, bool unal, const rl_launch_overrides& ov) {
-  const bool forced = ov.sweep_kernel >= 0 || ov.cluster_size > 0 || ov.cluster_stages > 0 ||
-                      ov.cluster_threads > 0 || ov.cluster_ctas_per_sm > 0 ||
-                      ov.stream_chunk_bytes > 0 || ov.stream_slots > 0 || ov.stream_hold >= 0 ||
-                      ov.stream_split_first >= 0 || ov.stream_prefetch_bytes >= 0 ||
-                      ov.stream_ctas_per_sm > 0 || ov.stream_cluster > 0 ||
-                      ov.stall_first_wait_ns > 0;
-  return !forced && !unal && row_bytes < kShortRowBytes;
+inline bool plan_forced(const rl_launch_overrides& ov) {
+  return ov.sweep_kernel >= 0 || ov.cluster_size > 0 || ov.cluster_stages > 0 ||
+         ov.cluster_threads > 0 || ov.cluster_ctas_per_sm > 0 ||
+         ov.stream_chunk_bytes > 0 || ov.stream_slots > 0 || ov.stream_hold >= 0 ||
+         ov.stream_split_first >= 0 || ov.stream_prefetch_bytes >= 0 ||
+         ov.stream_ctas_per_sm > 0 || ov.stream_cluster > 0 ||
+         ov.stall_first_wait_ns > 0;
 }
+inline bool use_short(long long row_bytes, bool unal, const rl_launch_overrides& ov) {
+  return !plan_forced(ov) && !unal && row_bytes < kShortRowBytes;
+}
+// Unaligned fp32 rows from this length on: k_stream in the cluster kernel's
+// order (4,096 rows of 4 KB: 60.4 us a call against 61.3, of 9 KB 66 against 92).
+constexpr long long kVirtRowBytes = 4 * 1024;
 // Warps per row and vectors per lane that hold a row of n_vec vectors.
 inline void short_shape(long long n_vec, int* warps, int* nv) {
   *warps = n_vec <= 512 ? 1 : (n_vec <= 1024 ? 2 : 4);

@@ -113,3 +113,36 @@ def test_unaligned_topk_and_vocab_shards():
     np.testing.assert_allclose(P.np_(shards[0].buf.token_logprobs), g["logp"], atol=tol, rtol=0)
     both = torch.cat([s.buf.dlogits for s in shards], 1).float().cpu().numpy()
     P.assert_dlogits_close(both, g["dlogits_t"].float().cpu().numpy())
+
+
+@pytest.mark.parametrize("vocab,off,topk", [
+    (1025, 0, 0), (3001, 1, 0), (10002, 2, 0), (18435, 3, 0), (20001, 0, 8), (20482, 1, 0),
+    (40001, 0, 0), (65539, 1, 0), (70001, 0, 0), (130003, 2, 0),
+])
+@pytest.mark.parametrize("mode", ["fused", "split"])
+def test_unaligned_fp32_keeps_the_cluster_kernels_sums(vocab, off, topk, mode):
+    """One, two, four and eight virtual slices, slices that end inside a
+    chunk, a row's last elements in a slice of their own: every output as the
+    cluster kernel has it."""
+    rec = wl.shrink(wl.RECIPES["fp32"], n_prompts=1, group_size=3, traj_len=37 if vocab < 9000 else 5,
+                    vocab=vocab, topk=topk)
+    w = wl.make(rec, DEV)
+    w.logits[1, :300] = -float("inf")
+    w.targets[1] = vocab - 1
+    w.logits[3, vocab // 2] = 120.0
+    w.targets[3] = vocab // 2
+    _, z = _offset(w.n_rows, vocab, off, torch.float32, float("nan"))
+    z.copy_(w.logits)
+    w = wl.Workload(**{**w.__dict__, "logits": z})
+    params = dict(w.params, **(dict(opd_topk=topk, opd_coef=0.4) if topk else {}))
+    got = P.run_gpu(w, mode=mode, params=params)
+    with ml.launch_overrides(sweep_kernel="cluster"):
+        want = P.run_gpu(w, mode=mode, params=params)
+    assert got["err"] == want["err"] == 0
+    if topk:  # (the candidates' parts merge in another order)
+        np.testing.assert_allclose(got["logp"], want["logp"], rtol=3e-7, atol=1e-6)
+        P.assert_dlogits_close(P.np_(got["dlogits_t"]), P.np_(want["dlogits_t"]))
+        return
+    np.testing.assert_array_equal(got["logp"], want["logp"])
+    np.testing.assert_array_equal(got["H"], want["H"])
+    assert torch.equal(got["dlogits_t"], want["dlogits_t"])
