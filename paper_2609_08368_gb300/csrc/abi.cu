@@ -658,11 +658,13 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
       st = plan_stream(dev, extra, row_bytes, static_cast<int>(es), grad, sc.topk > 0, unal,
                        f.part_rows == nullptr, pov, &sp);
       if (st != RL_OK) return st;
-      fn = stream_kernel(c.dt, grad ? go->dt : c.dt, grad, sc.topk > 0, unal, sp.cw, sp.cluster > 1);
+      const bool dec = stream_decoupled(row_bytes, grad, sc.topk > 0, unal, sp.cw);
+      fn = stream_kernel(c.dt, grad ? go->dt : c.dt, grad, sc.topk > 0, unal, sp.cw, sp.cluster > 1,
+                         dec);
       if (!fn) return RL_ERR_UNSUPPORTED;
       st = set_smem(fn, dev, sp.smem);
       if (st != RL_OK) return st;
-      threads = stream_threads(sc.topk > 0, sp.cw);
+      threads = stream_threads(sc.topk > 0, sp.cw, dec);
       st = resident_clusters(fn, dev, sp.cluster, sp.smem, threads, &ctas);
       // no cluster of the plan fits the device (a partition with too few SMs
       // together): one CTA per row instead, unless the override forced it

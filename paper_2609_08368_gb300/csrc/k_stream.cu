@@ -31,9 +31,9 @@ rl_status plan_stream(int dev, int extra, long long row_bytes, int es, bool grad
 }
 
 const void* stream_kernel(rl_dtype in, rl_dtype out, bool grad, bool topk, bool unal, int cw,
-                          bool clu) {
-  return unal ? stream_kernel_unal(in, out, grad, topk, cw, clu)
-              : pick_stream<false>(in, out, grad, topk, cw, clu);
+                          bool clu, bool dec) {
+  return unal ? stream_kernel_unal(in, out, grad, topk, cw, clu, dec)
+              : pick_stream<false>(in, out, grad, topk, cw, clu, dec);
 }
 
 }  // namespace milesloss

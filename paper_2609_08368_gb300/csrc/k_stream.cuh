@@ -261,8 +261,10 @@ __device__ __forceinline__ void pass_b_chunk(const uint4* sv, int nv, char* dchu
 // C times fewer rows are live at once, so a long row's second read still
 // comes from L2 (one CTA per SM keeps 152 rows live: 78 MB of 512 KB rows,
 // 304 MB of 2 MB rows, against a 126 MB L2).
-template <class In, class Out, bool kGrad, bool kTopK, int kCW, bool kClu, bool kUnal>
-__global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stream(const StreamArgs a) {
+template <class In, class Out, bool kGrad, bool kTopK, int kCW, bool kClu, bool kUnal, bool kDec>
+__global__ void __launch_bounds__(stream_threads(kTopK, kCW, kDec), 16 / kCW) k_stream(const StreamArgs a) {
+  // kDec (forward only): the epilogues run in a warp of their own (below)
+  static_assert(!kDec || !kGrad, "a pass B needs its row's epilogue");
   static_assert(!kClu || (kGrad && !kTopK && kCW == 16), "clusters: fused calls without top-K");
   constexpr int kCons = kCW * 32;  // consumer threads
   constexpr int kConsWarps = kCW;
@@ -318,9 +320,15 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
                         6 * 8 + 2 * 8 + 8 + 2 * kMaxCluster * 16 <=
                     kSweepSmemExtra,
                 "k_stream scratch");
+  // (kDec, which has no use for what else these hold) the warps' sums by row
+  // parity, with a "written" and a "read" barrier each
+  auto dec_red = [&](int b) { return b ? xch : red; };
+  uint64_t* dec_full = xbar;
+  uint64_t* dec_empty = reinterpret_cast<uint64_t*>(bc);
+  static_assert(kConsWarps <= 2 * kMaxCluster, "one parity's sums in xch");
   // (kUnal, fp32) the row's virtual slices (launched with kVirtSmem more): the
   // sums of each slice's eight warps
-  constexpr bool kVirt = kUnal && V8 == 4 && kCW == 8 && !kClu;
+  constexpr bool kVirt = kUnal && V8 == 4 && kCW == 8 && !kClu && !kDec;
   const bool virt = kVirt && a.virt_slice > 0;
   float4* vred = reinterpret_cast<float4*>(smem + static_cast<size_t>(NS) * CS + kSweepSmemExtra +
                                            (kTopK ? kTopKSmem : 0));
@@ -340,6 +348,12 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
     if (kClu) {
       mbar_init(smem_u32(&xbar[0]), 1);
       mbar_init(smem_u32(&xbar[1]), 1);
+    }
+    if (kDec) {
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(smem_u32(&dec_full[b]), kConsWarps);
+        mbar_init(smem_u32(&dec_empty[b]), 1);
+      }
     }
     *abort = 0;
     fence_mbar_init();
@@ -546,6 +560,106 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
     return;
   }
 
+  if (kDec && warp == kConsWarps + (kTopK ? 2 : 1)) {
+    // ------------------------------------------------- epilogues (forward only)
+    // No pass B waits for a row's epilogue, so the consumers go on to the next
+    // row at once: each warp leaves its sums in the buffer of the row's parity,
+    // and this warp merges them, in block_merge's order, and evaluates the row
+    // (its chain of logarithms, exponentials and stores is some 1 us, a fifth
+    // of a 40 KB row's time with four CTAs per SM). The target's logit comes
+    // from global memory, a row ahead. Calls before and after: 16,384 rows x
+    // 12,288 / 16,384 / 20,480 bf16 86 / 104 / 123 -> 74 / 93 / 113 us, 16,384 x
+    // 8,192 fp32 98 -> 90, 8,192 x 32,768 with top-K 110 -> 93.
+    float A = 0.0f, rho = 0.0f, q = 0.0f, old = 0.0f, zy = 0.0f;
+    int y = -1;
+    auto fetch = [&](long long row) {  // the row's inputs (lane 0)
+      const long long yl = a.targets[row] - a.col0;
+      y = (yl >= 0 && yl < a.V) ? static_cast<int>(yl) : -1;
+      rho = a.rho[row];
+      if (a.q) q = a.q[row];
+      if (a.old) old = a.old[row];
+      zy = y >= 0 ? In::load1(lg + row * a.ld * static_cast<long long>(sizeof(St)), y) : 0.0f;
+    };
+    if (lane == 0 && rows_mine > 0) fetch(cl_id);
+    for (long long i = 0; i < rows_mine; ++i) {
+      const long long row = cl_id + i * n_cl;
+      const int b = static_cast<int>(i & 1);
+      const bool yok = y >= 0;
+      const float rho_i = rho, q_i = q, old_i = old, zy_i = zy;
+      if (lane == 0 && i + 1 < rows_mine) fetch(row + n_cl);
+      if (i == 0) pdl_wait();  // the advantage kernel's results
+      if (lane == 0) A = ws.a_row[row];
+      const bool have = mbar_wait_or_abort(smem_u32(&dec_full[b]),
+                                           static_cast<uint32_t>((i >> 1) & 1), kWaitLimitNs,
+                                           abort, err);
+      Tri t{-INFINITY, 0.0f, 0.0f};
+      if (have) {
+        const float4* rb = dec_red(b);
+#pragma unroll
+        for (int w = 0; w < kCW; ++w) t.m = fmaxf(t.m, rb[w].x);
+        if (lane < kCW) {
+          const float4 v = rb[lane];
+          if (v.y > 0.0f) {
+            const float d = v.x - t.m, f = ex2(d);
+            t.s = f * v.y;
+            t.u = f * fmaf(d, v.y, v.z);
+          }
+        }
+#pragma unroll
+        for (int o = kCW / 2; o > 0; o >>= 1) {
+          t.s += __shfl_xor_sync(0xffffffffu, t.s, o);
+          t.u += __shfl_xor_sync(0xffffffffu, t.u, o);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&dec_empty[b]));
+      float opd = 0.0f;
+      int tk_bad = 0;
+      TopKPart part{-INFINITY, 0.0f, 0.0f, 0};
+      if (kTopK) {
+        if (mbar_wait_or_abort(smem_u32(&tk_full[b]), static_cast<uint32_t>((i >> 1) & 1),
+                               kWaitLimitNs, abort, err)) {
+          part = tkp[b];
+          opd = topk_value(part, fmaf(t.m, kLn2f, logf(t.s)));
+          tk_bad = part.bad;
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&tk_empty[b]));
+      }
+      if (lane != 0) continue;
+      if (a.part_rows) {
+        a.part_rows[2 * row] = *abort ? make_float4(NAN, 0.0f, 0.0f, 0.0f)
+                                      : make_float4(t.m, t.s, t.u, yok ? zy_i : 0.0f);
+        a.part_rows[2 * row + 1] = make_float4(part.m, part.sw, part.acc, part.bad ? 1.0f : 0.0f);
+        continue;
+      }
+      const bool bad = !yok || tk_bad || *abort;
+      const float lnS = logf(t.s);
+      const float lse = fmaf(t.m, kLn2f, lnS);
+      float H = lnS - t.u * kLn2f / t.s;
+      float logp = zy_i * a.s.invT - lse;
+      if (bad) { logp = 0.0f; H = 0.0f; }
+      if (a.s.topk > 0 && !bad) A -= a.s.opd_coef * opd;
+      TokenTerms tt = token_terms(logp, H, rho_i, q_i, a.q != nullptr, old_i, a.old != nullptr, A, a.s);
+      if (bad) tt = TokenTerms{0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, kFlagBad};
+      if (!yok) atomicOr(err, kErrTarget);
+      if (tk_bad) atomicOr(err, kErrTopK);
+      if (a.out_logp) a.out_logp[row] = logp;
+      if (a.out_H) a.out_H[row] = H;
+      ws.logp[row] = logp;
+      ws.H[row] = H;
+      ws.lse[row] = lse;
+      ws.G[row] = tt.G;
+      ws.ell[row] = tt.ell;
+      ws.pg[row] = tt.pg;
+      ws.k3[row] = tt.k3;
+      ws.r[row] = tt.r;
+      ws.rc[row] = tt.rc;
+      ws.flags[row] = tt.flags;
+    }
+    return;
+  }
+
   // -------------------------------------------------------------- consumers
   float cscale = 0.0f;  // (thread 0, from its first row's epilogue on)
   const float2 k2 = make_float2(k, k);
@@ -601,7 +715,7 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
     float rho = 0.0f, q = 0.0f, old = 0.0f, A = 0.0f, zy = 0.0f;
     uint8_t msk = 0;
     bool yok = false;
-    if (tid == 0) {
+    if (!kDec && tid == 0) {
       // the target's column in this call's logits (-1 outside them: a bad
       // target, or another shard's column in a vocabulary-sharded call)
       const long long yl = a.targets[row] - a.col0;
@@ -734,6 +848,20 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
         add1(kUnal ? z_tail : In::load1(grow, j));  // (kUnal: at most one per thread)
     }
 
+    if constexpr (kDec) {
+      t = warp_merge(t);
+      if (lane == 0) {
+        const int b = static_cast<int>(i & 1);
+        if (i >= 2)  // the sums of row i - 2 (same buffer) have been read
+          mbar_wait_or_abort(smem_u32(&dec_empty[b]), static_cast<uint32_t>(((i >> 1) - 1) & 1),
+                             kWaitLimitNs, abort, err);
+        dec_red(b)[warp] = make_float4(t.m, t.s, t.u, 0.0f);
+        mbar_arrive(smem_u32(&dec_full[b]));
+      }
+      __syncwarp();
+      q0 += n_chunks;
+      continue;
+    }
     if (i == 0 && tid == 0) {
       // the advantage kernel's results: it may still be running until here
       pdl_wait();
@@ -1004,6 +1132,7 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
     }
     q0 += (kGrad && trains) ? 2 * n_chunks - h : n_chunks;
   }
+  if constexpr (kDec) return;
   cons_sync<kCW>();
   if (tid == 0 && fix_ptr) Out::store1(fix_ptr, 0, fix_val);
   if constexpr (kClu) {  // no CTA leaves while a peer's last exchange store into it may be in flight
@@ -1012,35 +1141,45 @@ __global__ void __launch_bounds__(kCW * 32 + (kTopK ? 64 : 32), 16 / kCW) k_stre
   }
 }
 
+template <class In, class Out, bool kGrad, bool kUnal, int kCW>
+const void* fn_cw(bool topk, bool dec) {
+  if constexpr (!kGrad && !kUnal) {
+    if (dec && topk)
+      return reinterpret_cast<const void*>(&k_stream<In, Out, false, true, kCW, false, false, true>);
+    if constexpr (kCW == 4) {
+      if (dec)
+        return reinterpret_cast<const void*>(&k_stream<In, Out, false, false, 4, false, false, true>);
+    }
+  }
+  return topk ? reinterpret_cast<const void*>(&k_stream<In, Out, kGrad, true, kCW, false, kUnal, false>)
+              : reinterpret_cast<const void*>(&k_stream<In, Out, kGrad, false, kCW, false, kUnal, false>);
+}
+
+// dec as stream_decoupled gives it
 template <class In, class Out, bool kGrad, bool kUnal>
-const void* fn(bool topk, int cw, bool clu) {
+const void* fn(bool topk, int cw, bool clu, bool dec) {
   if constexpr (kGrad) {
     if (clu)
       return topk ? nullptr
-                  : reinterpret_cast<const void*>(&k_stream<In, Out, true, false, 16, true, kUnal>);
+                  : reinterpret_cast<const void*>(&k_stream<In, Out, true, false, 16, true, kUnal, false>);
   } else {
     if (clu) return nullptr;
   }
-  if (cw == 4)
-    return topk ? reinterpret_cast<const void*>(&k_stream<In, Out, kGrad, true, 4, false, kUnal>)
-                : reinterpret_cast<const void*>(&k_stream<In, Out, kGrad, false, 4, false, kUnal>);
-  if (cw == 8)
-    return topk ? reinterpret_cast<const void*>(&k_stream<In, Out, kGrad, true, 8, false, kUnal>)
-                : reinterpret_cast<const void*>(&k_stream<In, Out, kGrad, false, 8, false, kUnal>);
-  return topk ? reinterpret_cast<const void*>(&k_stream<In, Out, kGrad, true, 16, false, kUnal>)
-              : reinterpret_cast<const void*>(&k_stream<In, Out, kGrad, false, 16, false, kUnal>);
+  if (cw == 4) return fn_cw<In, Out, kGrad, kUnal, 4>(topk, dec);
+  if (cw == 8) return fn_cw<In, Out, kGrad, kUnal, 8>(topk, dec);
+  return fn_cw<In, Out, kGrad, kUnal, 16>(topk, dec);
 }
 
 template <bool kUnal>
-const void* pick_stream(rl_dtype in, rl_dtype out, bool grad, bool topk, int cw, bool clu) {
+const void* pick_stream(rl_dtype in, rl_dtype out, bool grad, bool topk, int cw, bool clu, bool dec) {
   if (!grad)
-    return in == RL_BF16 ? fn<InBf16, OutBf16, false, kUnal>(topk, cw, clu)
-                         : fn<InF32, OutF32, false, kUnal>(topk, cw, clu);
+    return in == RL_BF16 ? fn<InBf16, OutBf16, false, kUnal>(topk, cw, clu, dec)
+                         : fn<InF32, OutF32, false, kUnal>(topk, cw, clu, dec);
   if (in == RL_BF16)
-    return out == RL_BF16 ? fn<InBf16, OutBf16, true, kUnal>(topk, cw, clu)
-                          : fn<InBf16, OutF32, true, kUnal>(topk, cw, clu);
-  return out == RL_BF16 ? fn<InF32, OutBf16, true, kUnal>(topk, cw, clu)
-                        : fn<InF32, OutF32, true, kUnal>(topk, cw, clu);
+    return out == RL_BF16 ? fn<InBf16, OutBf16, true, kUnal>(topk, cw, clu, dec)
+                          : fn<InBf16, OutF32, true, kUnal>(topk, cw, clu, dec);
+  return out == RL_BF16 ? fn<InF32, OutBf16, true, kUnal>(topk, cw, clu, dec)
+                        : fn<InF32, OutF32, true, kUnal>(topk, cw, clu, dec);
 }
 
 }  // namespace

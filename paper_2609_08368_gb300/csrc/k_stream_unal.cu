@@ -4,8 +4,9 @@
 
 namespace milesloss {
 
-const void* stream_kernel_unal(rl_dtype in, rl_dtype out, bool grad, bool topk, int cw, bool clu) {
-  return pick_stream<true>(in, out, grad, topk, cw, clu);
+const void* stream_kernel_unal(rl_dtype in, rl_dtype out, bool grad, bool topk, int cw, bool clu,
+                               bool dec) {
+  return pick_stream<true>(in, out, grad, topk, cw, clu, dec);
 }
 
 }  // namespace milesloss

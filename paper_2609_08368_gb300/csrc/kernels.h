@@ -22,7 +22,19 @@ constexpr int kBwdThreads = 256;
 // k_stream's block: cw consumer warps (16 with one CTA per SM, 8 with two, 4
 // with four),
 // the producer warp and, with top-K OPD, the top-K warp
-constexpr int stream_threads(bool topk, int cw) { return cw * 32 + (topk ? 64 : 32); }
+// and, where it is decoupled, the epilogue warp: forward-only calls on aligned
+// rows, with four CTAs per SM up to 64 KB (calls without / with it: 64 KB rows
+// 91.7 / 90.7 us, 80 KB 107.8 / 109.8, 112 KB 143.6 / 148.6, unaligned 56 KB rows
+// 113 / 123: the fourth part of an SM's registers is tight for a sixth warp), and
+// with fewer where top-K OPD makes the epilogue longer (without top-K equal:
+// 8,192 x 65,536 167 / 163, but in a split call of 6,144 rows 343 / 351).
+inline bool stream_decoupled(long long row_bytes, bool grad, bool topk, bool unal, int cw) {
+  if (grad || unal) return false;
+  return cw == 4 ? row_bytes <= 64 * 1024 : topk;
+}
+__host__ __device__ constexpr int stream_threads(bool topk, int cw, bool dec) {
+  return cw * 32 + (topk ? 64 : 32) + (dec ? 32 : 0);
+}
 constexpr int kShortThreads = 128;
 constexpr int kSeqThreads = 256;
 constexpr int kAdvSmemBytes = 48 * 1024;  // on-chip trajectory tables when they fit
@@ -230,8 +242,9 @@ const void* short_kernel_topk(rl_dtype in, rl_dtype out, bool grad, int warps, i
 // calls without top-K only; nullptr otherwise)
 // unal: the instantiations for rows that do not all start on a 16-byte boundary
 const void* stream_kernel(rl_dtype in, rl_dtype out, bool grad, bool topk, bool unal, int cw,
-                          bool clu);
-const void* stream_kernel_unal(rl_dtype in, rl_dtype out, bool grad, bool topk, int cw, bool clu);
+                          bool clu, bool dec);
+const void* stream_kernel_unal(rl_dtype in, rl_dtype out, bool grad, bool topk, int cw, bool clu,
+                               bool dec);
 
 // The process-wide launch-plan overrides set by rl_set_launch_overrides (a
 // copy; every field -1 when none are set).
