@@ -20,12 +20,17 @@
 // same), with its fixed orders of merging. The eight warps' butterfly sums
 // share their shuffles (at each step a lane keeps half of the values and sends
 // the other half, which adds the same pairs).
-// Measured against k_sweep, whole calls: 2,048 x 4,096 bf16 28.3 -> 22.8 us in a
-// graph; 32,768 rows x 2,048 / 4,096 / 9,600 bf16 179 / 198 / 248 -> 74 / 121 /
-// 233; 65,536 x 8,192 435 -> 406; 32,768 x 4,096 fp32 230 -> 200; forward only,
-// 32,768 x 4,096 / 8,192 bf16 156 / 174 -> 76 / 122.
+// Instruction issue bounds it (19 warp instructions per 32 logits and some 950 a
+// row, 62 % of the issue slots, before the usual sums skipped the floor, a
+// row's mode was chosen outside pass B and the rescale had one test: 32,768
+// rows x 2,048 / 4,096 / 9,600 72.6 / 119 / 229 -> 68.4 / 112 / 220 us).
+// Measured against k_sweep, whole calls: 32,768 rows x 2,048 / 4,096 / 9,600 bf16
+// 179 / 198 / 248 -> 68 / 112 / 220 us; 65,536 x 8,192 435 -> 364; 32,768 x 4,096
+// fp32 230 -> 176; forward only, 32,768 x 4,096 / 8,192 bf16 156 / 174 -> 71 / 116.
 // Definitions: Sec. 3.4 (ratio), Sec. 2 / 9.1 (advantage), Sec. 2.4 (mask).
 #pragma once
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -155,7 +160,9 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
   const float k = a.s.k;
   const float2 k2 = make_float2(k, k);
   float vm[kJ], vs[kJ], vu[kJ];
-  auto sums = [&](int j, float r, float& s, float& u) {  // against the reference r
+  // against the reference r; safe: logits far below any that matter taken at
+  // the floor (the usual sums skip that)
+  auto sums = [&](auto safe, int j, float r, float& s, float& u) {
     const float2 nr2 = make_float2(-r, -r);
     float2 s0 = make_float2(0.0f, 0.0f), s1 = s0, u0 = s0, u1 = s0;
 #pragma unroll
@@ -163,7 +170,7 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
       const int i = j + kJ * ii;
       if (i < kNV && i * kT + t < n_vec) {
         float2 f[P];
-        In::unpack2(FloorOf<In>::apply(raw[i]), f);
+        In::unpack2(decltype(safe)::value ? FloorOf<In>::apply(raw[i]) : raw[i], f);
 #pragma unroll
         for (int e = 0; e < P; ++e) {
           const float2 x2 = ffma2(f[e], k2, nr2), x = ex2x2(x2);
@@ -181,19 +188,19 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
     s = s2.x + s2.y;
     u = u2.x + u2.y;
   };
-  uint32_t redo = 0;  // threads whose first vector's maximum does not serve
+  uint32_t redo = 0;  // threads whose sums are not finite
 #pragma unroll
   for (int j = 0; j < kJ; ++j) {
     vm[j] = -INFINITY;
     vs[j] = vu[j] = 0.0f;
     if (j * kT + t < n_vec) {
       const float r = In::vmax(raw[j]) * k;
-      sums(j, r, vs[j], vu[j]);
+      sums(std::false_type{}, j, r, vs[j], vu[j]);
       vm[j] = r;
       if (!(fabsf(vs[j]) < INFINITY) || !(fabsf(vu[j]) < INFINITY) || r == -INFINITY) redo |= 1u << j;
     }
   }
-  if (redo) {  // (rare: an overflow, or a first vector of -inf) the thread's own maximum
+  if (redo) {  // (rare: an overflow, or a -inf logit) the thread's own maximum
 #pragma unroll
     for (int j = 0; j < kJ; ++j) {
       if (!(redo >> j & 1u)) continue;
@@ -205,18 +212,22 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
       }
       vm[j] = In::max_val(macc) * k;
       vs[j] = vu[j] = 0.0f;
-      if (vm[j] != -INFINITY) sums(j, vm[j], vs[j], vu[j]);
+      if (vm[j] != -INFINITY) sums(std::true_type{}, j, vm[j], vs[j], vu[j]);
     }
   }
+  float most = vs[0];
 #pragma unroll
-  for (int j = 0; j < kJ; ++j) {
-    // sums past 2^16 move the reference up by their binary exponent
-    const int e = ((__float_as_int(vs[j]) >> 23) & 0xff) - 127;
-    if (e > 16) {
-      const float f = __int_as_float((127 - e) << 23), d = static_cast<float>(e);
-      vu[j] = f * fmaf(-d, vs[j], vu[j]);
-      vs[j] *= f;
-      vm[j] += d;
+  for (int j = 1; j < kJ; ++j) most = fmaxf(most, vs[j]);
+  if (most >= 131072.0f) {  // sums past 2^16 move the reference up by their binary exponent
+#pragma unroll
+    for (int j = 0; j < kJ; ++j) {
+      const int e = ((__float_as_int(vs[j]) >> 23) & 0xff) - 127;
+      if (e > 16) {
+        const float f = __int_as_float((127 - e) << 23), d = static_cast<float>(e);
+        vu[j] = f * fmaf(-d, vs[j], vu[j]);
+        vs[j] *= f;
+        vm[j] += d;
+      }
     }
   }
   if (has_tail && z_tail != -INFINITY) {  // (the block's first threads: j = 0 of warp 0)
@@ -334,34 +345,42 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
                            : cc * (tt.G * -expm1f(logp) + a.s.gamma * expf(logp) * (logp + H));
     const float2 off2 = make_float2(off, off), ca2 = make_float2(ca, ca), cb2 = make_float2(cb, cb);
     const float sgn = (fold && ca < 0.0f) ? -1.0f : 1.0f;
-    const float2 sgn2 = make_float2(sgn, sgn);
     const int yv = yok ? y / V8 : -1;
+    // mode 0: p |ca|, 1: -p |ca|, 2: p (ca + cb z), 3: zeros
+    auto pass_b = [&](auto mode) {
+      constexpr int kMode = decltype(mode)::value;
 #pragma unroll
-    for (int i = 0; i < kNV; ++i) {
-      const int v = i * kT + t;
-      if (v < n_vec) {
-        float2 f[P];
-        if (zero) {
+      for (int i = 0; i < kNV; ++i) {
+        const int v = i * kT + t;
+        if (v < n_vec) {
+          float2 f[P];
+          if (kMode == 3) {
 #pragma unroll
-          for (int e = 0; e < P; ++e) f[e] = make_float2(0.0f, 0.0f);
-        } else {
-          In::unpack2(raw[i], f);
+            for (int e = 0; e < P; ++e) f[e] = make_float2(0.0f, 0.0f);
+          } else {
+            In::unpack2(raw[i], f);
 #pragma unroll
-          for (int e = 0; e < P; ++e) {
-            const float2 p = ex2x2(ffma2(f[e], k2, off2));
-            f[e] = fmul2(p, fold ? sgn2 : ent_factor2(f[e], ca2, cb2));
+            for (int e = 0; e < P; ++e) {
+              const float2 p = ex2x2(ffma2(f[e], k2, off2));
+              if (kMode == 2) f[e] = fmul2(p, ent_factor2(f[e], ca2, cb2));
+              else f[e] = kMode == 1 ? make_float2(-p.x, -p.y) : p;
+            }
+            if (v == yv) {
+              float* fv = reinterpret_cast<float*>(f);
+#pragma unroll
+              for (int e = 0; e < V8; ++e)
+                if (v * V8 + e == y) fv[e] = dzy;
+            }
           }
-          if (v == yv) {
-            float* fv = reinterpret_cast<float*>(f);
-#pragma unroll
-            for (int e = 0; e < V8; ++e)
-              if (v * V8 + e == y) fv[e] = dzy;
-          }
+          Out::template storev<V8>(drow + static_cast<size_t>(v) * V8 * Out::kSize,
+                                   reinterpret_cast<const float*>(f), 0u);
         }
-        Out::template storev<V8>(drow + static_cast<size_t>(v) * V8 * Out::kSize,
-                                 reinterpret_cast<const float*>(f), 0u);
       }
-    }
+    };
+    if (zero) pass_b(std::integral_constant<int, 3>{});
+    else if (!fold) pass_b(std::integral_constant<int, 2>{});
+    else if (ca < 0.0f) pass_b(std::integral_constant<int, 1>{});
+    else pass_b(std::integral_constant<int, 0>{});
     if (has_tail) {
       float x = 0.0f;
       if (!zero) x = ex2(fmaf(z_tail, k, off)) * (fold ? sgn : ent_factor(z_tail, ca, cb));
