@@ -506,6 +506,7 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
   // alone: then the kernels run one after the other.
   const bool overlap = !(t_ev_begin && t_ev_end);
   bool pdl = false;  // the call has launched a kernel
+  bool small_smem = false;  // the sweep is k_short
 
   if (phase & RL_PHASE_BEGIN) {
   const Common& c = call;
@@ -645,6 +646,7 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     record(t_ev_end, s);
     if (st != RL_OK) return st;
     pdl = overlap;
+    small_smem = true;
   } else if (c.R > 0 && stream) {
     const void* fn = nullptr;
     int ctas = 0;  // resident CTAs, or clusters of sp.cluster CTAs
@@ -765,16 +767,21 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     pdl = overlap;
   }
 
+  // GSPO's gradient, from the trajectories' terms. After a sweep that fills the
+  // shared memory it is no dependent: its blocks would start on SMs still set
+  // up for that, with 28 KB of L1 for their loads in flight (8,192 x 151,936
+  // bf16: 1,225 us that way, 1,080 before any kernel overlapped).
+  if (gspo && go && (phase & RL_PHASE_ROWS) && call.R > 0) {
+    st = launch_bwd(call, *go, ws_all, s, 0, pdl && small_smem);
+    if (st != RL_OK) return st;
+    pdl = overlap;
+  }
+
   if ((phase & RL_PHASE_END) && (f.stats || f.part_out)) {
     st = launch_stats(f, f.stats, f.part_out, s, pdl);
     if (st != RL_OK) return st;
     pdl = overlap;
   }
-  // (Not as a dependent: its blocks would start on SMs still set up for the
-  // sweep's shared memory, with 28 KB of L1 for their loads in flight. GSPO,
-  // 8,192 x 151,936 bf16: 1,225 us that way, 1,080 before any kernel overlapped.)
-  if (gspo && go && (phase & RL_PHASE_ROWS) && call.R > 0)
-    return launch_bwd(call, *go, ws_all, s, 0, false);
   return RL_OK;
 }
 
@@ -945,12 +952,12 @@ rl_status rl_loss_shard_fwd_bwd(int32_t phase, int64_t row_offset, int64_t n_row
     st = launch_seq(f, nullptr, traj_sums, s, false);
     if (st != RL_OK) return st;
   }
-  st = launch_stats(f, nullptr, partials, s, n_traj > 0);
-  if (st != RL_OK) return st;
-  if (grad && n_rows > 0)
-    return launch_bwd(f.c, go, WsPtrs::at(workspace, WsLayout::make(n_rows, n_traj, n_groups)), s,
-                      0, true);
-  return RL_OK;
+  if (grad && n_rows > 0) {
+    st = launch_bwd(f.c, go, WsPtrs::at(workspace, WsLayout::make(n_rows, n_traj, n_groups)), s, 0,
+                    n_traj > 0);
+    if (st != RL_OK) return st;
+  }
+  return launch_stats(f, nullptr, partials, s, n_traj > 0 || (grad && n_rows > 0));
 }
 
 rl_status rl_loss_vocab_shard_fwd_bwd(
@@ -1041,10 +1048,11 @@ rl_status rl_loss_vocab_shard_fwd_bwd(
       st = launch_seq(f, nullptr, traj_sums, s, false);
       if (st != RL_OK) return st;
     }
-    st = launch_stats(f, nullptr, partials, s, n_traj > 0);
-    if (st != RL_OK) return st;
-    if (grad && n_rows > 0) return launch_bwd(f.c, go, ws, s, col0, true);
-    return RL_OK;
+    if (grad && n_rows > 0) {
+      st = launch_bwd(f.c, go, ws, s, col0, n_traj > 0);
+      if (st != RL_OK) return st;
+    }
+    return launch_stats(f, nullptr, partials, s, n_traj > 0 || (grad && n_rows > 0));
   }
   if (n_rows > 0) {
     int dev = 0, sms = 0;
