@@ -37,7 +37,7 @@ METRIC = "RL-loss fwd+bwd tokens/sec at vocab 154,880 bf16; achieved HBM GB/s vs
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6800.0
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "stream_kernel_glm.md")
-SWEEP_SOURCES = ["k_stream.cu", "stream_plan.h", "common.cuh", "kernels.h"]  # the kernel and its launch plan
+SWEEP_SOURCES = ["k_stream.cuh", "k_stream.cu", "stream_plan.h", "common.cuh", "kernels.h"]  # the kernel and its launch plan
 
 
 def parse_args():
@@ -283,11 +283,21 @@ def sweep_kernel_name(vocab: int, elem_size: int, grad: bool = True, topk: bool 
     return f"k_sweep ({kind} vocabulary sweep, clusters sharing a row)"
 
 
-def launches_per_call(params: dict, n_groups: int) -> int:
-    """Kernels one fused call launches: group statistics (when there are
-    groups), advantages, the sweep and the statistics; GSPO adds the
-    per-trajectory pass and the gradient sweep."""
-    n = 3 + (1 if n_groups > 8 else 0)  # up to 8 groups, k_advantages computes them itself
+def sweep_kernel_label(vocab: int, elem_size: int, grad: bool = True, topk: bool = False,
+                       forced: str | None = None, forced_cluster: int | None = None) -> str:
+    """sweep_kernel_name, or the short-row kernel, which takes (aligned) rows
+    below 20 KB from the cluster kernel when nothing is forced."""
+    if vocab * elem_size < 20 * 1024 and not forced and not forced_cluster:
+        kind = "fused fwd+bwd" if grad else "forward-only"
+        return f"k_short ({kind} vocabulary sweep, a row in the registers of one to four warps)"
+    return sweep_kernel_name(vocab, elem_size, grad, topk, forced, forced_cluster)
+
+
+def launches_per_call(params: dict, n_groups: int, n_traj: int = 1 << 15) -> int:
+    """Kernels one fused call launches: advantages, the sweep and the
+    statistics, with many groups and trajectories the group statistics
+    before them; GSPO adds the per-trajectory pass and the gradient sweep."""
+    n = 3 + (1 if n_groups * n_traj > 1 << 20 else 0)
     return n + (2 if params.get("estimator", "grpo") == "gspo" else 0)
 
 
@@ -798,16 +808,16 @@ def run_ours(args, rank, world, local):
     also["split_fwd_bwd_tokens_per_s"] = R / (also["split_fwd_bwd_ms"] / 1e3)
 
     bpr = algorithmic_bytes_per_row(w, dl_dtype)  # before w is released for the e2e leg
-    kernel_name = sweep_kernel_name(V, w.logits.element_size(), topk=bool(args.opd_topk),
+    kernel_name = sweep_kernel_label(V, w.logits.element_size(), topk=bool(args.opd_topk),
                                     forced=args.sweep_kernel, forced_cluster=args.stream_cluster)
-    w_params, n_groups = dict(w.params), w.n_groups
+    w_params, n_groups, n_traj = dict(w.params), w.n_groups, int(w.rewards.shape[0])
     step_bytes = bpr * R
     launch_bytes = step_bytes
     if w_params.get("estimator", "grpo") == "gspo":
         # GSPO's timed sweep is the forward-only one (k_seq and the gradient
         # sweep k_bwd follow it): it reads the logits and writes no dLogits
         launch_bytes = (bpr - V * torch.tensor([], dtype=dl_dtype).element_size()) * R
-        kernel_name = sweep_kernel_name(V, w.logits.element_size(), grad=False,
+        kernel_name = sweep_kernel_label(V, w.logits.element_size(), grad=False,
                                         topk=bool(args.opd_topk), forced=args.sweep_kernel) + \
             ", GSPO's first pass (k_bwd reads the logits again for dLogits)"
     sweep_avg = statistics.fmean(sweep_ms)
@@ -890,7 +900,7 @@ def run_ours(args, rank, world, local):
         "also": also,
         "cpu_baseline": cpu,
         "e2e": e2e,
-        "gpu_launches": launches_per_call(w_params, n_groups) * K,
+        "gpu_launches": launches_per_call(w_params, n_groups, n_traj) * K,
         "clocks": clk,
         "loss": stats["loss"],
     }

@@ -651,8 +651,10 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     const void* fn = nullptr;
     int ctas = 0;  // resident CTAs, or clusters of sp.cluster CTAs
     int threads = 0;
+    // unaligned logits: the cluster kernel's slices (fp32 rows are summed by
+    // them), and its limit on a row's length
     SweepPlan slices{};
-    if (virt) {
+    if (!in_bulk) {
       st = plan_sweep(c.dt, c.V, dev, sc.topk ? kTopKSmem : 0, grad, ov, &slices);
       if (st != RL_OK) return st;
     }

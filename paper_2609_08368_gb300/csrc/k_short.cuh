@@ -23,9 +23,9 @@
 // Instruction issue bounds it (19 warp instructions per 32 logits and some 950 a
 // row, 62 % of the issue slots, before the usual sums skipped the floor, a
 // row's mode was chosen outside pass B and the rescale had one test: 32,768
-// rows x 2,048 / 4,096 / 9,600 72.6 / 119 / 229 -> 68.4 / 112 / 220 us).
+// rows x 2,048 / 4,096 / 9,600 73.1 / 120 / 231 -> 68.3 / 110 / 222 us).
 // Measured against k_sweep, whole calls: 32,768 rows x 2,048 / 4,096 / 9,600 bf16
-// 179 / 198 / 248 -> 68 / 112 / 220 us; 65,536 x 8,192 435 -> 364; 32,768 x 4,096
+// 179 / 198 / 248 -> 68 / 110 / 222 us; 65,536 x 8,192 435 -> 366; 32,768 x 4,096
 // fp32 230 -> 176; forward only, 32,768 x 4,096 / 8,192 bf16 156 / 174 -> 71 / 116.
 // Definitions: Sec. 3.4 (ratio), Sec. 2 / 9.1 (advantage), Sec. 2.4 (mask).
 #pragma once
@@ -346,7 +346,11 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
     const float2 off2 = make_float2(off, off), ca2 = make_float2(ca, ca), cb2 = make_float2(cb, cb);
     const float sgn = (fold && ca < 0.0f) ? -1.0f : 1.0f;
     const int yv = yok ? y / V8 : -1;
-    // mode 0: p |ca|, 1: -p |ca|, 2: p (ca + cb z), 3: zeros
+    // mode 0: p |ca| with ca's sign, 1: p (ca + cb z), 2: zeros. (The two signs
+    // share their code: a small call fetches each form's instructions once per
+    // SM, and rows of both signs meet there; a third form cost 2,048 x 4,096
+    // in a graph 18.5 -> 20.8 us.)
+    const float2 sgn2 = make_float2(sgn, sgn);
     auto pass_b = [&](auto mode) {
       constexpr int kMode = decltype(mode)::value;
 #pragma unroll
@@ -354,7 +358,7 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
         const int v = i * kT + t;
         if (v < n_vec) {
           float2 f[P];
-          if (kMode == 3) {
+          if (kMode == 2) {
 #pragma unroll
             for (int e = 0; e < P; ++e) f[e] = make_float2(0.0f, 0.0f);
           } else {
@@ -362,8 +366,7 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
 #pragma unroll
             for (int e = 0; e < P; ++e) {
               const float2 p = ex2x2(ffma2(f[e], k2, off2));
-              if (kMode == 2) f[e] = fmul2(p, ent_factor2(f[e], ca2, cb2));
-              else f[e] = kMode == 1 ? make_float2(-p.x, -p.y) : p;
+              f[e] = fmul2(p, kMode == 1 ? ent_factor2(f[e], ca2, cb2) : sgn2);
             }
             if (v == yv) {
               float* fv = reinterpret_cast<float*>(f);
@@ -377,10 +380,9 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
         }
       }
     };
-    if (zero) pass_b(std::integral_constant<int, 3>{});
-    else if (!fold) pass_b(std::integral_constant<int, 2>{});
-    else if (ca < 0.0f) pass_b(std::integral_constant<int, 1>{});
-    else pass_b(std::integral_constant<int, 0>{});
+    if (zero) pass_b(std::integral_constant<int, 2>{});
+    else if (fold) pass_b(std::integral_constant<int, 0>{});
+    else pass_b(std::integral_constant<int, 1>{});
     if (has_tail) {
       float x = 0.0f;
       if (!zero) x = ex2(fmaf(z_tail, k, off)) * (fold ? sgn : ent_factor(z_tail, ca, cb));
