@@ -51,8 +51,9 @@
 // other's (virt_slice), from the slots. (A log-prob's last bit, where a token's
 // gradient is the difference to its reference's, is 2e-4 of a dLogit.)
 // Fused calls, against that kernel: 4,096 rows x 5,001 / 10,001 / 32,769 147 /
-// 237 / 667 -> 82 / 133 / 373 us, 2,048 x 130,003 2,085 -> 581, 1,024 x 230,003
-// 5,447 -> 567; the chain of a running maximum bounds it.
+// 237 / 667 -> 65 / 98 / 266 us, 2,048 x 130,003 2,085 -> 426, 1,024 x 230,003
+// 5,447 -> 406; the chain of a running maximum bounds it (with that kernel's
+// branches 82 / 133 / 373, 581, 567).
 // Definitions: Sec. 3.4 (ratio), Sec. 2 / 9.1 (advantage), Sec. 2.4 (mask).
 #pragma once
 
@@ -760,6 +761,33 @@ __global__ void __launch_bounds__(stream_threads(kTopK, kCW, kDec), 16 / kCW) k_
     };
     if constexpr (kVirt) {
       if (virt) {
+        // add1 without its branches, which a warp's lanes take at nearly every
+        // element of a 73-element slice: the rescale runs each time, by
+        // 2^0 = 1 when the maximum stays (exact), the products rounded as
+        // add1's are (not fused); a -inf logit adds nothing at kVirtFloor,
+        // and a reference below that stands for "none yet".
+        constexpr float kVirtFloor = -1.0e30f, kVirtNone = -2.0e38f;
+        float m = kVirtNone, s = 0.0f, u = 0.0f;
+        auto add = [&](float z) {
+          float zf;  // max(z, floor), NaN kept
+          asm("max.NaN.f32 %0, %1, %2;" : "=f"(zf) : "f"(z), "f"(kVirtFloor));
+          const float mn = fmaxf(m, zf * k);
+          const float d = m - mn, f = ex2(d);
+          // (at the floor the product's rounding error is 1e22, not below 1)
+          float tt = fmaf(zf, k, -mn);
+          asm("min.NaN.f32 %0, %0, %1;" : "+f"(tt) : "f"(1.0f));
+          const float x = ex2(tt);
+          u = fmaf(x, tt, __fmul_rn(f, fmaf(d, s, u)));
+          s = __fadd_rn(__fmul_rn(s, f), x);
+          m = mn;
+        };
+        auto sums = [&]() {  // the thread's slice; a new one starts
+          const bool none = m < -1.0e29f * k;  // nothing but -inf, or no element
+          const Tri r{none ? -INFINITY : m, none ? 0.0f : s, none ? 0.0f : u};
+          m = kVirtNone;
+          s = u = 0.0f;
+          return r;
+        };
         int vc = 0;
         for (int c = 0; c < n_chunks; ++c) {
           wait_slot(q0 + c);
@@ -772,18 +800,18 @@ __global__ void __launch_bounds__(stream_threads(kTopK, kCW, kDec), 16 / kCW) k_
             const int lo = vc * a.virt_slice;
             const int end = vc == a.virt_c - 1 ? e1 : min(e1, lo + a.virt_slice);
 #pragma unroll 4
-            for (int j = e0 + ((tid - (e0 - lo)) & 255); j < end; j += 256) add1(src[j]);
+            for (int j = e0 + ((tid - (e0 - lo)) & 255); j < end; j += 256) add(src[j]);
             e0 = end;
             if (vc < a.virt_c - 1 && end == lo + a.virt_slice) {  // the slice is complete
-              t = warp_merge(t);
+              t = warp_merge(sums());
               if (lane == 0) vred[vc * 8 + warp] = make_float4(t.m, t.s, t.u, 0.0f);
-              t = Tri{-INFINITY, 0.0f, 0.0f};
               ++vc;
             }
           }
           if (c < n_chunks - h) release_slot(q0 + c);
         }
-        if (j_tail < a.V) add1(z_tail);
+        if (j_tail < a.V) add(z_tail);
+        t = sums();
       }
     }
     for (int c = virt ? n_chunks : 0; c < n_chunks; ++c) {

@@ -103,7 +103,7 @@ inline bool use_short(long long row_bytes, bool unal, const rl_launch_overrides&
   return !plan_forced(ov) && !unal && row_bytes < kShortRowBytes;
 }
 // Unaligned fp32 rows from this length on: k_stream in the cluster kernel's
-// order (4,096 rows of 4 KB: 60.4 us a call against 61.3, of 9 KB 66 against 92).
+// order (4,096 rows of 4 KB: 57 us a call against 61, of 9 KB 59 against 92).
 constexpr long long kVirtRowBytes = 4 * 1024;
 // Warps per row and vectors per lane that hold a row of n_vec vectors.
 inline void short_shape(long long n_vec, int* warps, int* nv) {

@@ -146,3 +146,19 @@ def test_unaligned_fp32_keeps_the_cluster_kernels_sums(vocab, off, topk, mode):
     np.testing.assert_array_equal(got["logp"], want["logp"])
     np.testing.assert_array_equal(got["H"], want["H"])
     assert torch.equal(got["dlogits_t"], want["dlogits_t"])
+
+
+@pytest.mark.parametrize("dtype,vocab", [("f32", 10001), ("bf16", 20001)])
+def test_unaligned_nan_stays_in_its_row(dtype, vocab):
+    """A NaN logit reaches its own dLogit (as in an aligned row) and no other
+    row's outputs."""
+    rec = wl.shrink(wl.RECIPES["fp32" if dtype == "f32" else "glm"], n_prompts=1, group_size=2,
+                    traj_len=6, vocab=vocab, mask="none")
+    w = wl.make(rec, DEV)
+    clean = P.run_gpu(w)
+    w.logits[5, 777] = float("nan")
+    got = P.run_gpu(w)
+    rest = [r for r in range(w.n_rows) if r != 5]
+    np.testing.assert_array_equal(got["logp"][rest], clean["logp"][rest])
+    assert torch.isnan(got["dlogits_t"][5, 777])
+    assert torch.equal(got["dlogits_t"][rest], clean["dlogits_t"][rest])
