@@ -48,7 +48,7 @@ struct StatPart {
 constexpr int kMaxTopK = 64;
 constexpr int kStatThreads = 256;
 constexpr int kStatCluster = 8;      // up to this many blocks run as one cluster
-constexpr int kMaxStatBlocks = 256;  // one partial per thread of the final block
+constexpr int kMaxStatBlocks = 256;
 
 struct WsLayout {
   size_t hdr, g_mu, g_den, g_flag, a_traj, traj_n, a_row;

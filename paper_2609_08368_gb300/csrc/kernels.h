@@ -255,7 +255,8 @@ rl_status status_of_bits(uint32_t bits);
 // The streaming kernel's launch plan (k_stream.cu, from the pure plan in
 // stream_plan.h): whether rows of row_bytes go to it, and its ring of
 // shared-memory slots.
-// (unal: the rows of the logits or of dLogits do not all start on a 16-byte boundary)
+// (in_bulk: every row of the logits starts on a 16-byte boundary; unal: not
+// every row of the logits and of dLogits does)
 bool use_stream(long long row_bytes, int es, bool in_bulk, bool unal, bool grad, bool topk,
                 const rl_launch_overrides& ov);
 // extra: shared memory beyond the ring and the fixed scratch (kTopKSmem with
