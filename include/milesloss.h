@@ -504,7 +504,8 @@ const char* rl_status_string(rl_status status);
 /* Launch-plan overrides: measurement aids and a test hook, not needed for
  * normal use. The library picks every launch shape itself (the sweep kernel
  * by row length, the cluster kernel's cluster size, ring depth and block
- * shape, the streaming kernel's ring); these fields force one instead. -1
+ * shape, the streaming kernel's ring); these fields force one instead (and
+ * any of them takes rows below 20 KB from the short-row kernel). -1
  * in a field keeps the library's choice; rl_launch_overrides_init sets
  * every field to -1. A forced value outside the compiled shapes makes later
  * calls return RL_ERR_UNSUPPORTED before anything is enqueued.

@@ -280,8 +280,9 @@ __device__ __forceinline__ void cluster_sync_all() {
 // dependent of the one before it in the stream may start once every CTA of
 // that kernel has called pdl_trigger (or has exited); pdl_wait then waits
 // until that kernel has finished and its writes are visible. The first kernel
-// of a call is an ordinary launch, or (advantages) a dependent of whatever ran
-// before that waits for it before anything else, its own trigger included: so
+// of a call is an ordinary launch, or (advantages, a chunked call's sweep) a
+// dependent of whatever ran before that waits for it before anything else,
+// its own trigger included: so
 // nothing of an earlier call, or of the caller's, is still running when the
 // call's other kernels start. Each of those calls pdl_wait before it reads or
 // writes anything that an earlier kernel of the call touches: inputs of the

@@ -273,6 +273,7 @@ __global__ void __launch_bounds__(stream_threads(kTopK, kCW, kDec), 16 / kCW) k_
   constexpr int V8 = In::kVec;
   constexpr int P = V8 / 2;
   extern __shared__ __align__(128) unsigned char smem[];
+  if (a.first) pdl_wait();
   pdl_trigger();
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;

@@ -86,6 +86,8 @@ struct StreamArgs {
   int n_hold;       // last chunks of a row that pass B reads from shared memory (<= n_slots)
   int split_first;  // 1: the first chunk takes the ragged remainder (rounded up to 128 bytes)
   int prefetch;     // bytes of the next row to ask L2 for once a row's first pass is issued
+  int first;        // the call's first kernel, launched as a dependent all the same: it waits
+                    // for what ran before the call, before anything else
   int virt_slice;   // > 0: unaligned fp32 rows, summed as virt_c slices of this many
   int virt_c;       // elements are by the cluster kernel (k_stream.cuh)
   int slice_vec;    // launched in clusters (one per row): whole vectors of a row per CTA, a
