@@ -271,6 +271,17 @@ __device__ __forceinline__ uint32_t cluster_nctarank() {
   return r;
 }
 
+// A CTA may touch a peer's shared memory only once that peer is known to have
+// started: after a barrier of the cluster. cluster_arrive and a later
+// cluster_wait are one in two halves, for a kernel with other work meanwhile
+// (relaxed: it orders no memory, only the CTAs' starts). Every thread of every
+// CTA calls both.
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                "barrier.cluster.wait.acquire.aligned;" ::: "memory");

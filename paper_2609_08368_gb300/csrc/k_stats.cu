@@ -93,6 +93,12 @@ __global__ void __launch_bounds__(kStatThreads) k_stats(const StatArgs a) {
   __shared__ int s_last;
   WsPtrs ws = a.ws;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // one cluster of all the blocks (below): each must know that the first has
+  // started before it stores into its shared memory; the wait is after the
+  // rows' loads and costs nothing there
+  const int NC = static_cast<int>(cluster_nctarank());
+  const bool one_cluster = gridDim.x > 1 && static_cast<int>(gridDim.x) == NC;
+  if (one_cluster) cluster_arrive();
   pdl_trigger();
   pdl_wait();
   // 1 / N while the rows' loads are on their way (the rows' own count is the
@@ -135,6 +141,7 @@ __global__ void __launch_bounds__(kStatThreads) k_stats(const StatArgs a) {
     for (int i = 0; i < 5; ++i) sh_c[warp][kCount0 + i] = p.c[i];
   }
   __syncthreads();
+  if (one_cluster) cluster_wait();
   // the block's results: thread q < 16 merges the warps' result q, in order
   const int q = tid & (kStatFields - 1);
   const bool is_count = q >= kCount0 && q < kMin;
@@ -152,8 +159,7 @@ __global__ void __launch_bounds__(kStatThreads) k_stats(const StatArgs a) {
       mine = static_cast<double>(v);
     }
   }
-  const int NC = static_cast<int>(cluster_nctarank());
-  if (gridDim.x > 1 && static_cast<int>(gridDim.x) == NC) {
+  if (one_cluster) {
     // one cluster: every block's results into the first block's shared memory
     const uint32_t rank = cluster_ctarank();
     if (tid < kStatFields)
