@@ -548,12 +548,19 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     st = launch(groups_kernel(), dim3(static_cast<unsigned>(gb)), dim3(32), 0, 1, s, &aa, early);
     if (st != RL_OK) return st;
   }
-  if (aa.estimator == RL_EST_GRPO && aa.smem_traj && !aa.groups_done && aa.n_traj > 0 &&
-      !aa.counts_out)
-    st = launch(adv_grpo_kernel(), dim3(adv_grpo_ctas(c.R, aa.n_traj)), dim3(kAdvThreads),
+  const bool grpo = aa.estimator == RL_EST_GRPO && aa.smem_traj && !aa.groups_done &&
+                    aa.n_traj > 0 && !aa.counts_out;
+  const void* fn = grpo ? adv_grpo_kernel() : adv_kernel();
+  // tables and static shared memory together may pass the default 48 KB
+  if (aa.smem_traj && traj_bytes > 48 * 1024 - static_cast<size_t>(kAdvStaticBytes)) {
+    st = set_smem(fn, dev, kAdvSmemBytes);
+    if (st != RL_OK) return st;
+  }
+  if (grpo)
+    st = launch(fn, dim3(adv_grpo_ctas(c.R, aa.n_traj)), dim3(kAdvThreads),
                 static_cast<int>(traj_bytes), 1, s, &aa, early);
   else
-    st = launch(adv_kernel(), dim3(kAdvCluster), dim3(kAdvThreads),
+    st = launch(fn, dim3(kAdvCluster), dim3(kAdvThreads),
                 aa.smem_traj ? static_cast<int>(traj_bytes) : 0, kAdvCluster, s, &aa, early);
   if (st != RL_OK) return st;
   pdl = overlap;

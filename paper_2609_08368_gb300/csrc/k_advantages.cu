@@ -159,6 +159,8 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_advantages(const AdvArgs a) 
   __shared__ double s_red[kMergeMax][kWarps + 1];
   __shared__ unsigned long long s_tok;
   __shared__ unsigned int s_seq;
+  static_assert(sizeof(s_err) + sizeof(s_red) + sizeof(s_tok) + sizeof(s_seq) + 64 <= kAdvStaticBytes,
+                "static shared memory beside the tables");
   WsPtrs ws = a.ws;
   // Shared copies, when they fit, of cu (n_traj + 1), group ids and rewards,
   // and the advantages of this CTA's trajectories.
@@ -434,6 +436,8 @@ __global__ void __launch_bounds__(kAdvThreads, 1) k_adv_grpo(const AdvArgs a) {
   const int nt = a.n_traj;
   __shared__ unsigned int s_err;
   __shared__ unsigned int s_cnt[kWarps];
+  static_assert(sizeof(s_err) + sizeof(s_cnt) + 64 <= kAdvStaticBytes,
+                "static shared memory beside the tables");
   int* cu = dyn;
   int* gid = dyn + (nt + 1);
   float* rew = reinterpret_cast<float*>(dyn + (2 * nt + 1));

@@ -38,6 +38,9 @@ __host__ __device__ constexpr int stream_threads(bool topk, int cw, bool dec) {
 constexpr int kShortThreads = 128;
 constexpr int kSeqThreads = 256;
 constexpr int kAdvSmemBytes = 48 * 1024;  // on-chip trajectory tables when they fit
+// The advantage kernels' own (static) shared memory, at most (asserted there).
+// It counts towards the 48 KB that a launch gets unasked.
+constexpr int kAdvStaticBytes = 1024;
 constexpr int kVirtSmem = kMaxCluster * 8 * 16;     // the warps' sums of a row's virtual slices
 constexpr int kTopKSmem = 2 * (2 * kMaxTopK * 4);  // two rows of top-K ids + teacher values
 

@@ -35,3 +35,23 @@ def test_grpo_advantages(n_prompts, group, traj_len, opd):
     np.testing.assert_array_equal(g["group_sizes"], o["group_sizes"])
     assert g["stats"]["n_tokens"] == int(w.loss_mask.sum())
     P.assert_dlogits_close(g["dlogits_t"].float().cpu().numpy(), o["dlogits"])
+
+
+@pytest.mark.parametrize("estimator", ["grpo", "reinforcepp_baseline", "gspo"])
+@pytest.mark.parametrize("n_prompts,group", [
+    (1, 3007), (1, 3008), (1, 3044), (1, 3045), (1, 3066), (1, 3067),
+    (1, 3071), (1, 3072),                            # the last tables of 48 KB, the first past them
+    (381, 8), (383, 8),                              # group statistics in a kernel of their own
+])
+def test_trajectory_tables_at_the_shared_memory_limit(n_prompts, group, estimator):
+    """A launch that asks for nothing has 48 KB for the tables and the kernel's
+    own shared memory together."""
+    rec = wl.shrink(wl.RECIPES["tiny"], n_prompts=n_prompts, group_size=group, traj_len=1, vocab=16,
+                    reward="normal", mask="none")
+    w = wl.make(rec, DEV)
+    params = dict(w.params, estimator=estimator)
+    g, o = P.run_gpu(w, params=params), P.run_oracle(w, params=params)
+    assert g["err"] == 0
+    np.testing.assert_allclose(g["A"], o["A_traj"], rtol=1e-6, atol=1e-7)
+    np.testing.assert_array_equal(g["group_sizes"], o["group_sizes"])
+    P.assert_dlogits_close(g["dlogits_t"].float().cpu().numpy(), o["dlogits"])
