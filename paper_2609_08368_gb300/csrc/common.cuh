@@ -190,6 +190,32 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
   }
 }
 
+// Programmatic dependent launch. A kernel launched as a programmatic
+// dependent of the one before it in the stream may start once every CTA of
+// that kernel has called pdl_trigger (or has exited); pdl_wait then waits
+// until that kernel has finished and its writes are visible. The first kernel
+// of a call is an ordinary launch, or (advantages, a chunked call's sweep) a
+// dependent of whatever ran before that waits for it before anything else,
+// its own trigger included: so
+// nothing of an earlier call, or of the caller's, is still running when the
+// call's other kernels start. Each of those calls pdl_wait before it reads or
+// writes anything that an earlier kernel of the call touches: inputs of the
+// call may be read before it. (Without the launch attribute both are no-ops.)
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Records a wait that ran out. The error word is one of the things that the
+// advantage kernel writes (it resets it), and a dependent's wait may run out
+// before that kernel has: hence the wait for it.
+__device__ __forceinline__ void record_timeout(uint32_t* err) {
+  pdl_wait();
+  atomicOr(err, kErrTimeout);
+}
+
 // A CTA's shared "give up" flag: once one party of the CTA has given up on a
 // wait, the others stop waiting too (their next wait returns at once), so a
 // CTA that meets one timeout finishes in about one wait limit instead of one
@@ -224,7 +250,7 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint32_t bar, uint32_t parity
       }
       if (globaltimer_ns() - t0 > limit_ns) {
         *abort = 1;
-        atomicOr(err, kErrTimeout);
+        record_timeout(err);
         return false;
       }
     }
@@ -285,24 +311,6 @@ __device__ __forceinline__ void cluster_wait() {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// Programmatic dependent launch. A kernel launched as a programmatic
-// dependent of the one before it in the stream may start once every CTA of
-// that kernel has called pdl_trigger (or has exited); pdl_wait then waits
-// until that kernel has finished and its writes are visible. The first kernel
-// of a call is an ordinary launch, or (advantages, a chunked call's sweep) a
-// dependent of whatever ran before that waits for it before anything else,
-// its own trigger included: so
-// nothing of an earlier call, or of the caller's, is still running when the
-// call's other kernels start. Each of those calls pdl_wait before it reads or
-// writes anything that an earlier kernel of the call touches: inputs of the
-// call may be read before it. (Without the launch attribute both are no-ops.)
-__device__ __forceinline__ void pdl_trigger() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {

@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(stream_threads(kTopK, kCW, kDec), 16 / kCW) k_
           const long long last = q - 1 - ((q - 1 - s) % NS);
           if (!mbar_wait_bounded(smem_u32(&full[s]), static_cast<uint32_t>((last / NS) & 1),
                                  kWaitLimitNs))
-            atomicOr(err, kErrTimeout);
+            record_timeout(err);
         }
       }
     }
@@ -964,7 +964,7 @@ __global__ void __launch_bounds__(stream_threads(kTopK, kCW, kDec), 16 / kCW) k_
           if (!mbar_wait_bounded(xb, static_cast<uint32_t>((i >> 1) & 1), kWaitLimitNs)) {
             xdead = true;
             *abort = 1;
-            atomicOr(err, kErrTimeout);
+            record_timeout(err);
           }
         }
         float M = -INFINITY;

@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep(const SweepArgs 
           if (!mbar_wait_bounded(xb, static_cast<uint32_t>((it >> 1) & 1), kWaitLimitNs)) {
             xdead = true;
             *abort = 1;
-            atomicOr(err, kErrTimeout);
+            record_timeout(err);
           }
         }
         float M = -INFINITY;
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep(const SweepArgs 
     for (int s = 0; s < S; ++s)
       if ((iss_any & (1u << s)) &&
           !mbar_wait_bounded(smem_u32(&bars[s]), ((iss_par >> s) & 1u) ^ 1u, kWaitLimitNs))
-        atomicOr(err, kErrTimeout);
+        record_timeout(err);
   }
   // No CTA leaves while a peer's last exchange store into it may be in flight.
   if (C > 1) cluster_sync_all();
