@@ -174,19 +174,29 @@ def _dtype_code(t) -> int:
     return code
 
 
-_torch = None
+_raw_stream = None
+
+
+def _raw_stream_of(torch):
+    """A function for the current stream's handle. torch's own C entry points
+    give it without a Stream object (2.8 us a call); where a torch has not got
+    them, its public interface does."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    dev = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or dev is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(dev())
 
 
 def _stream(stream):
     if stream is not None:
         return stream.cuda_stream
-    global _torch
-    if _torch is None:
+    global _raw_stream
+    if _raw_stream is None:
         import torch
         torch.cuda.current_stream()  # (initialises CUDA in a process that has not yet)
-        _torch = torch
-    # torch.cuda.current_stream().cuda_stream without the Stream object (2.8 us)
-    return _torch._C._cuda_getCurrentRawStream(_torch._C._cuda_getDevice())
+        _raw_stream = _raw_stream_of(torch)
+    return _raw_stream()
 
 
 def rl_loss_workspace_size(n_rows: int, n_traj: int, n_groups: int) -> int:

@@ -335,3 +335,15 @@ def test_vocab_sharded_entry_validates(lib):
     tk = ml.make_params(opd_coef=0.5, opd_topk=4)                      # no candidate arrays
     assert call(PA, params=tk) == RL_ERR_INVALID_ARG
     assert call(PA, params=ml.make_params(temperature=0.0)) == RL_ERR_INVALID_ARG
+
+
+def test_current_stream_with_and_without_torchs_own_entry_points():
+    """The stream of a call that names none: torch's C entry points where they
+    exist, its public interface where they do not."""
+    from types import SimpleNamespace as NS
+    public = NS(current_stream=lambda: NS(cuda_stream=17))
+    own = NS(_cuda_getDevice=lambda: 3, _cuda_getCurrentRawStream=lambda dev: 100 + dev)
+    assert ml._raw_stream_of(NS(_C=own, cuda=public))() == 103
+    assert ml._raw_stream_of(NS(_C=NS(), cuda=public))() == 17
+    del own._cuda_getDevice
+    assert ml._raw_stream_of(NS(_C=own, cuda=public))() == 17
