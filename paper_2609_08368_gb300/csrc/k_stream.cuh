@@ -330,8 +330,11 @@ __global__ void __launch_bounds__(stream_threads(kTopK, kCW, kDec), 16 / kCW) k_
   static_assert(kConsWarps <= 2 * kMaxCluster, "one parity's sums in xch");
   // (kUnal, fp32) the row's virtual slices (launched with kVirtSmem more): the
   // sums of each slice's eight warps
+  // (in a fused call the logits may be aligned and only dLogits not: then no
+  // slices, and no shift; a forward-only call is here for its logits)
   constexpr bool kVirt = kUnal && V8 == 4 && kCW == 8 && !kClu && !kDec;
-  const bool virt = kVirt && a.virt_slice > 0;
+  const bool virt = kVirt && (!kGrad || a.virt_slice > 0);
+  constexpr bool kShift = kUnal && V8 == 8;  // pass A reads vectors through the row's shift
   float4* vred = reinterpret_cast<float4*>(smem + static_cast<size_t>(NS) * CS + kSweepSmemExtra +
                                            (kTopK ? kTopKSmem : 0));
   // [2] top-K candidates of this row and the next (launched with kTopKSmem more)
@@ -821,7 +824,7 @@ __global__ void __launch_bounds__(stream_threads(kTopK, kCW, kDec), 16 / kCW) k_
       const int v0 = cs(c), nv = cn(c);
       {
         if (tid == 0 && yv >= v0 && yv < v0 + nv) zy = In::load1(sv, y - (lo_v + v0) * V8 + sh);
-        auto vec_at = [&](int v) { return kUnal ? shifted_any<In>(sv, v, sh) : sv[v]; };
+        auto vec_at = [&](int v) { return kShift ? shifted_any<In>(sv, v, sh) : sv[v]; };
         if (run.r == -INFINITY && tid < nv) run.raise(In::vmax(vec_at(tid)) * k);
         const Run keep = run;
         bool redo = run.r == -INFINITY;  // no finite reference yet
@@ -836,9 +839,9 @@ __global__ void __launch_bounds__(stream_threads(kTopK, kCW, kDec), 16 / kCW) k_
                                                               (e & 1) ? run.u1 : run.u0);
             }
           };
-          if constexpr (kUnal) {
-            const uint32_t hs = (V8 == 8 && (sh & 1)) ? 16u : 0u;
-            switch (V8 == 8 ? sh >> 1 : sh) {
+          if constexpr (kShift) {
+            const uint32_t hs = (sh & 1) ? 16u : 0u;
+            switch (sh >> 1) {
               case 0:
                 if (hs == 0) sum_chunk([&](int v) { return sv[v]; });
                 else sum_chunk([&](int v) { return shifted<0>(sv, v, hs); });
@@ -1194,9 +1197,11 @@ const void* fn(bool topk, int cw, bool clu, bool dec) {
   } else {
     if (clu) return nullptr;
   }
-  if (cw == 4) return fn_cw<In, Out, kGrad, kUnal, 4>(topk, dec);
   if (cw == 8) return fn_cw<In, Out, kGrad, kUnal, 8>(topk, dec);
-  return fn_cw<In, Out, kGrad, kUnal, 16>(topk, dec);
+  // (unaligned fp32 logits: virtual slices, eight warps)
+  if constexpr (kUnal && !kGrad && In::kVec == 4) return nullptr;
+  else return cw == 4 ? fn_cw<In, Out, kGrad, kUnal, 4>(topk, dec)
+                      : fn_cw<In, Out, kGrad, kUnal, 16>(topk, dec);
 }
 
 template <bool kUnal>
