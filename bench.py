@@ -284,16 +284,34 @@ def sweep_kernel_name(vocab: int, elem_size: int, grad: bool = True, topk: bool 
 
 
 def sweep_kernel_label(vocab: int, elem_size: int, grad: bool = True, topk: bool = False,
-                       forced: str | None = None, forced_cluster: int | None = None) -> str:
-    """sweep_kernel_name, or the short-row kernel, which takes (aligned) rows
-    below 20 KB from the cluster kernel when nothing is forced."""
-    if vocab * elem_size < 20 * 1024 and not forced and not forced_cluster:
-        kind = "fused fwd+bwd" if grad else "forward-only"
+                       forced: str | None = None, forced_cluster: int | None = None,
+                       aligned: bool = True) -> str:
+    """sweep_kernel_name, and what it leaves out: with nothing forced, the
+    short-row kernel for rows below 20 KB, and for rows that do not all start
+    on a 16-byte boundary (in the logits and in dLogits alike: not
+    ``aligned``) the streaming kernel's unaligned forms: bf16 rows of any
+    length, fp32 rows from 4 KB on in the cluster kernel's slices."""
+    KB, row_bytes = 1024, vocab * elem_size
+    kind = "fused fwd+bwd" if grad else "forward-only"
+    if aligned and row_bytes < 20 * KB and not forced and not forced_cluster:
         return f"k_short ({kind} vocabulary sweep, a row in the registers of one to four warps)"
-    return sweep_kernel_name(vocab, elem_size, grad, topk, forced, forced_cluster)
+    if aligned or forced == "cluster":
+        return sweep_kernel_name(vocab, elem_size, grad, topk, forced, forced_cluster)
+    if elem_size == 4:
+        if forced or forced_cluster or row_bytes < 4 * KB:
+            return sweep_kernel_name(vocab, elem_size, grad, topk, forced="cluster")
+        return f"k_stream ({kind} vocabulary sweep, unaligned rows, one CTA per row, 2 CTAs per SM)"
+    # bf16: the tiers of aligned rows; where those have the cluster kernel, CTAs
+    # per SM by length
+    name = sweep_kernel_name(vocab, elem_size, grad, topk, forced_cluster=forced_cluster)
+    if name.startswith("k_sweep"):
+        per = 1 if grad and row_bytes >= 136 * KB else (2 if topk or row_bytes > 56 * KB else 4)
+        name = f"k_stream ({kind} vocabulary sweep, one CTA per row" + \
+            (f", {per} CTAs per SM)" if per > 1 else ")")
+    return name.replace("vocabulary sweep", "vocabulary sweep, unaligned rows")
 
 
-def launches_per_call(params: dict, n_groups: int, n_traj: int = 1 << 15) -> int:
+def launches_per_call(params: dict, n_groups: int, n_traj: int) -> int:
     """Kernels one fused call launches: advantages, the sweep and the
     statistics, with many groups and trajectories the group statistics
     before them; GSPO adds the per-trajectory pass and the gradient sweep."""
@@ -808,8 +826,11 @@ def run_ours(args, rank, world, local):
     also["split_fwd_bwd_tokens_per_s"] = R / (also["split_fwd_bwd_ms"] / 1e3)
 
     bpr = algorithmic_bytes_per_row(w, dl_dtype)  # before w is released for the e2e leg
+    aligned = all(t.data_ptr() % 16 == 0 and t.stride(0) * t.element_size() % 16 == 0
+                  for t in (w.logits, buf.dlogits))
     kernel_name = sweep_kernel_label(V, w.logits.element_size(), topk=bool(args.opd_topk),
-                                    forced=args.sweep_kernel, forced_cluster=args.stream_cluster)
+                                    forced=args.sweep_kernel, forced_cluster=args.stream_cluster,
+                                    aligned=aligned)
     w_params, n_groups, n_traj = dict(w.params), w.n_groups, int(w.rewards.shape[0])
     step_bytes = bpr * R
     launch_bytes = step_bytes
@@ -818,7 +839,8 @@ def run_ours(args, rank, world, local):
         # sweep k_bwd follow it): it reads the logits and writes no dLogits
         launch_bytes = (bpr - V * torch.tensor([], dtype=dl_dtype).element_size()) * R
         kernel_name = sweep_kernel_label(V, w.logits.element_size(), grad=False,
-                                        topk=bool(args.opd_topk), forced=args.sweep_kernel) + \
+                                        topk=bool(args.opd_topk), forced=args.sweep_kernel,
+                                        aligned=aligned) + \
             ", GSPO's first pass (k_bwd reads the logits again for dLogits)"
     sweep_avg = statistics.fmean(sweep_ms)
     peaks, peak_kind = measured_peaks()

@@ -17,10 +17,12 @@ from paper_2609_08368_gb300 import api, workloads as wl  # noqa: E402
 
 
 def test_launches_per_call():
-    assert bench.launches_per_call({}, 4) == 3                     # glm: groups inline
-    assert bench.launches_per_call({}, 64) == 4                    # fp32: k_groups too
-    assert bench.launches_per_call({"estimator": "gspo"}, 4) == 5  # + k_seq, k_bwd
-    assert bench.launches_per_call({"estimator": "reinforcepp"}, 1) == 3
+    assert bench.launches_per_call({}, 4, 64) == 3       # glm: groups inline
+    assert bench.launches_per_call({}, 64, 512) == 3     # fp32: inline too
+    assert bench.launches_per_call({}, 1024, 1024) == 3  # up to 2^20 pairs of group and trajectory
+    assert bench.launches_per_call({}, 1024, 1025) == 4  # past that k_groups
+    assert bench.launches_per_call({"estimator": "gspo"}, 4, 64) == 5  # + k_seq, k_bwd
+    assert bench.launches_per_call({"estimator": "reinforcepp"}, 1, 4) == 3
 
 
 def test_sweep_kernel_name_follows_the_plan_tiers():
@@ -71,6 +73,29 @@ def test_sweep_kernel_name_follows_the_plan_tiers():
     # the stream_cluster override (fused calls without top-K only)
     assert "a cluster of 4 CTAs per row" in bench.sweep_kernel_name(154880, 2, forced_cluster=4)
     assert bench.sweep_kernel_name(154880, 2, topk=True, forced_cluster=4).endswith(one)
+
+
+def test_sweep_kernel_label():
+    """Short and unaligned rows, which the tiers leave out."""
+    label = bench.sweep_kernel_label
+    assert label(4096, 2).startswith("k_short (fused")
+    assert label(10232, 2, grad=False).startswith("k_short (forward-only")
+    assert label(10240, 2) == bench.sweep_kernel_name(10240, 2)            # 20 KB
+    assert label(4096, 2, forced="cluster").startswith("k_sweep")
+    assert label(154880, 2) == bench.sweep_kernel_name(154880, 2)
+    unal, un = "k_stream (fused fwd+bwd vocabulary sweep, unaligned rows", dict(aligned=False)
+    assert label(1001, 2, **un) == unal + ", one CTA per row, 4 CTAs per SM)"
+    assert label(45003, 2, **un) == unal + ", one CTA per row, 2 CTAs per SM)"  # 88 KB
+    assert label(75003, 2, **un) == unal + ", one CTA per row)"             # 146 KB
+    assert label(154883, 2, **un) == unal + ", one CTA per row)"
+    assert label(250001, 2, **un) == unal + ", a cluster of 2 CTAs per row)"
+    assert label(8001, 2, topk=True, **un) == unal + ", one CTA per row, 2 CTAs per SM)"
+    assert label(45003, 2, forced="cluster", **un).startswith("k_sweep")
+    assert label(45003, 2, forced="stream", **un) == label(45003, 2, **un)
+    # fp32: the cluster kernel's slices, from 4 KB on and with nothing forced
+    assert label(32769, 4, **un) == unal + ", one CTA per row, 2 CTAs per SM)"
+    assert label(1001, 4, **un).startswith("k_sweep")
+    assert label(32769, 4, forced="stream", **un).startswith("k_sweep")
 
 
 def test_profiled_traffic_only_for_its_workload_and_sources():
