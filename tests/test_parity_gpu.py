@@ -625,6 +625,28 @@ def test_a_wait_that_runs_out_is_reported(ov, kind, topk):
         _full_check(w, mode=mode, params=params)
 
 
+@pytest.mark.parametrize("stall_ns", [1, 1_000_000])
+@pytest.mark.parametrize("name,vocab,topk", [
+    ("glm", 12288, 0), ("glm", 28672, 0), ("fp32", 8192, 0),    # four CTAs per SM
+    ("glm", 40960, 4), ("glm", 110000, 4)])                      # two, one
+def test_a_forward_only_wait_that_runs_out_is_reported(ov, name, vocab, topk, stall_ns):
+    """The same for forward-only calls, whose epilogues run in a warp of their
+    own on rows up to 64 KB (with top-K on rows of any length), with several
+    rows to a CTA."""
+    rec = wl.shrink(wl.RECIPES[name], n_prompts=1, group_size=4, traj_len=600 if topk == 0 else 100,
+                    vocab=vocab, rho_noise=0.3, topk=topk, topk_noise=0.4)
+    w = wl.make(rec, DEV)
+    params = dict(w.params, opd_coef=0.5, opd_topk=topk) if topk else None
+    ov(stall_first_wait_ns=stall_ns)
+    g = P.run_gpu(w, mode="fwd", params=params)
+    assert g["err"] == 8, ml.status_string(g["err"])  # RL_ERR_DEVICE_TIMEOUT
+    assert np.all(g["logp"] == 0) and np.all(g["H"] == 0)
+    st = g["stats"]
+    assert st["loss"] == 0.0 and st["n_tokens"] == int(w.loss_mask.sum())
+    ov(stall_first_wait_ns=-1)
+    _full_check(w, mode="fwd", params=params)
+
+
 @pytest.mark.parametrize("kind,cluster", [("cluster", 0), ("cluster", 4), ("stream", 0)])
 def test_topk_ids_out_of_range_are_reported(ov, kind, cluster):
     """A top-K OPD candidate id outside [0, vocab) zeros its row (as a bad

@@ -1,5 +1,5 @@
 """A host model of the streaming sweep kernel's shared-memory ring protocol
-(csrc/k_stream.cu), checked without a GPU.
+(csrc/k_stream.cuh), checked without a GPU.
 
 Four parties share the ring: the producer issues one bulk copy per task into
 slot task % n_slots once every reader has released the task n_slots before;
@@ -203,7 +203,13 @@ class _Barrier:
 
 class _GiveUpSim:
     def __init__(self, masks, n, grad, NS, hold, topk, fail_site=None, stall=False, seed=0,
-                 n_cons=2):
+                 n_cons=2, dec=False):
+        assert not (dec and grad)  # an epilogue warp: forward-only calls
+        self.dec = dec
+        self.dec_full = [_Barrier(n_cons), _Barrier(n_cons)]
+        self.dec_empty = [_Barrier(1), _Barrier(1)]
+        self.dec_sums = [{}, {}]  # buffer -> consumer warp -> row its sums belong to
+        self.rows_out = {}        # row -> taken as good
         self.masks, self.n, self.grad, self.NS, self.hold, self.topk = masks, n, grad, NS, hold, topk
         self.rng = random.Random(seed)
         self.tasks = list(producer_tasks(masks, n, grad, hold))
@@ -266,6 +272,14 @@ class _GiveUpSim:
                     yield ("read", me, q, self.tasks[q])
                 if c < n - h:
                     yield ("release", me, q)
+            if self.dec:
+                b = i & 1
+                if i >= 2:
+                    yield ("wait", self.dec_empty[b], (i >> 1) - 1, True, (me, "dec_empty"))
+                yield ("dec_write", b, me, i)
+                yield ("arrive", self.dec_full[b])
+                q0 += n
+                continue
             gen = yield ("sync_arrive", me)
             yield ("sync_wait", gen)
             if self.topk and warp0:
@@ -310,9 +324,23 @@ class _GiveUpSim:
             q0 += 2 * n - h if trains else n
         yield ("done", "T")
 
+    def epilogue_warp(self):
+        for i in range(len(self.masks)):
+            b = i & 1
+            ok = yield ("wait", self.dec_full[b], i >> 1, True, ("E", "dec_full"))
+            seen = yield ("dec_read", b) if ok else ("dec_skip",)
+            yield ("arrive", self.dec_empty[b])
+            if self.topk:
+                yield ("wait", self.tk_full[b], i >> 1, True, ("E", "tk_full"))
+                yield ("arrive", self.tk_empty[b])
+            yield ("row_out", i, seen)
+        yield ("done", "E")
+
     # ---- scheduler
     def run(self):
         gens = {"P": self.producer()}
+        if self.dec:
+            gens["E"] = self.epilogue_warp()
         for k, r in enumerate(r for r in self.readers if r != "T"):
             gens[r] = self.consumer(r, warp0=(k == 0))
         if self.topk:
@@ -369,6 +397,18 @@ class _GiveUpSim:
                 self.empty[q % self.NS].arrive()
             elif kind == "arrive":
                 r[1].arrive()
+            elif kind == "dec_write":
+                self.dec_sums[r[1]][r[2]] = r[3]
+            elif kind == "dec_read":
+                res = dict(self.dec_sums[r[1]])
+            elif kind == "row_out":
+                # the CTA's flag is read after the sums: with it up the row is
+                # zeros, else its sums are those of every warp for this row
+                _, i, seen = r
+                if not self.abort:
+                    assert seen is not None and set(seen.values()) == {i} and \
+                        len(seen) == self.dec_full[0].count, f"row {i} from sums of {seen}"
+                self.rows_out[i] = not self.abort
             elif kind == "sync_arrive":
                 g = self.sync_gen.get(r[1], 0)
                 self.sync_gen[r[1]] = g + 1
@@ -385,7 +425,8 @@ class _GiveUpSim:
                 if kind in ("done", "producer_done"):
                     done.add(name)
                     continue
-                req[name] = gens[name].send(res if kind in ("wait", "sync_arrive") else None)
+                req[name] = gens[name].send(res if kind in ("wait", "sync_arrive", "dec_read")
+                                            else None)
                 self.flag_seen[name] = self.abort
             except StopIteration:
                 done.add(name)
@@ -418,9 +459,9 @@ class _GiveUpSim:
         return None
 
 
-def _sites(masks, n, grad, NS, hold, topk):
+def _sites(masks, n, grad, NS, hold, topk, dec=False):
     """Every wait site an uninterrupted run passes, with its ordinal."""
-    sim = _GiveUpSim(masks, n, grad, NS, hold, topk, seed=1).run()
+    sim = _GiveUpSim(masks, n, grad, NS, hold, topk, seed=1, dec=dec).run()
     return [(site, k) for site, cnt in sim.wait_count.items() if site[0] != "P" or
             site[1] == "empty" for k in range(cnt)]
 
@@ -448,6 +489,54 @@ def test_give_up_at_every_wait(grad, topk):
                     sim = _GiveUpSim(masks, n, grad, NS, hold, topk, stall=True, seed=seed).run()
                     assert sim.failed and sim.producer_done
     assert cases > 100
+
+
+@pytest.mark.parametrize("topk", [False, True])
+def test_give_up_with_an_epilogue_warp(topk):
+    """Forward-only calls with the epilogues in a warp of their own: the
+    consumer warps leave a row's sums in the buffer of its parity, once the
+    epilogue warp has read those of two rows before, and go on."""
+    rng = random.Random(13)
+    cases = 0
+    for n in (1, 2, 4):
+        for NS in (1, 2, 3):
+            masks = [rng.random() < 0.7 for _ in range(rng.randint(1, 7))]
+            for seed in range(20):
+                sim = _GiveUpSim(masks, n, False, NS, 0, topk, seed=seed, dec=True).run()
+                assert sim.rows_out == {i: True for i in range(len(masks))}
+            for site in _sites(masks, n, False, NS, 0, topk, dec=True):
+                for seed in range(6):
+                    sim = _GiveUpSim(masks, n, False, NS, 0, topk, fail_site=site, seed=seed,
+                                     dec=True).run()
+                    assert sim.failed and sim.producer_done and len(sim.rows_out) == len(masks)
+                    cases += 1
+            for seed in range(6):
+                sim = _GiveUpSim(masks, n, False, NS, 0, topk, stall=True, seed=seed, dec=True).run()
+                assert sim.failed and sim.producer_done
+    assert cases > 100
+
+
+def test_model_catches_sums_overwritten_before_they_are_read():
+    class Hasty(_GiveUpSim):
+        def consumer(self, me, warp0):
+            g = _GiveUpSim.consumer(self, me, warp0)
+            r = next(g)
+            while True:
+                if r[0] == "wait" and r[4][1] == "dec_empty":
+                    r = g.send(True)
+                    continue
+                res = yield r
+                try:
+                    r = g.send(res)
+                except StopIteration:
+                    return
+    caught = 0
+    for seed in range(50):
+        try:
+            Hasty([True] * 6, 1, False, 3, 0, False, seed=seed, dec=True).run()
+        except AssertionError:
+            caught += 1
+    assert caught > 0
 
 
 def _producer_without(sim, skip):
