@@ -507,6 +507,7 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
   const bool overlap = !(t_ev_begin && t_ev_end);
   bool pdl = false;  // the call has launched a kernel
   bool small_smem = false;  // the sweep is k_short
+  int adv_ctas = 0;  // CTAs of the call's advantage kernel
 
   if (phase & RL_PHASE_BEGIN) {
   const Common& c = call;
@@ -556,12 +557,10 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     st = set_smem(fn, dev, kAdvSmemBytes);
     if (st != RL_OK) return st;
   }
-  if (grpo)
-    st = launch(fn, dim3(adv_grpo_ctas(c.R, aa.n_traj)), dim3(kAdvThreads),
-                static_cast<int>(traj_bytes), 1, s, &aa, early);
-  else
-    st = launch(fn, dim3(kAdvCluster), dim3(kAdvThreads),
-                aa.smem_traj ? static_cast<int>(traj_bytes) : 0, kAdvCluster, s, &aa, early);
+  adv_ctas = grpo ? adv_grpo_ctas(c.R, aa.n_traj) : kAdvCluster;
+  st = launch(fn, dim3(adv_ctas), dim3(kAdvThreads),
+              aa.smem_traj ? static_cast<int>(traj_bytes) : 0, grpo ? 1 : kAdvCluster, s, &aa,
+              early);
   if (st != RL_OK) return st;
   pdl = overlap;
   }
@@ -740,6 +739,15 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     st = resident_clusters(fn, dev, pl.C, pl.smem, pl.threads, &clusters);
     if (st != RL_OK) return st;
     const long long n_cl = std::min<long long>(clusters, c.R);
+    // Clusters of four that fill the GPU are no dependents: those that find no
+    // four free places beside the advantage kernel's CTAs get theirs only when
+    // others have swept all their rows. It takes more than three such CTAs, and
+    // costs more than the overlap gives from some four rows a cluster on. As a
+    // dependent / not (us), 64 trajectories, 190 clusters: 128 rows x 65,792
+    // 16 / 22, 512 40 / 40, 704 51 / 51, 768 57 / 53, 1,024 72 / 64, 4,096 255 /
+    // 197; 8 trajectories (three CTAs) 1,024 59 / 63, 4,096 195 / 197; 8,192 x
+    // 90,112 664 / 483. Clusters of two: 4,096 x 60,000 175 / 181.
+    const bool beside = pl.C < 4 || c.R <= 4LL * clusters || adv_ctas <= 3;
 
     SweepArgs sa;
     sa.logits = c.logits;
@@ -770,7 +778,7 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     sa.part_rows = shift(f.part_rows, 2 * r0);
     record(t_ev_begin, s);
     st = launch(fn, dim3(static_cast<unsigned>(n_cl * pl.C)), dim3(pl.threads), pl.smem, pl.C,
-                s, &sa, pdl);
+                s, &sa, pdl && beside);
     record(t_ev_end, s);
     if (st != RL_OK) return st;
     pdl = overlap;
