@@ -313,9 +313,11 @@ def sweep_kernel_label(vocab: int, elem_size: int, grad: bool = True, topk: bool
 
 def launches_per_call(params: dict, n_groups: int, n_traj: int) -> int:
     """Kernels one fused call launches: advantages, the sweep and the
-    statistics, with many groups and trajectories the group statistics
-    before them; GSPO adds the per-trajectory pass and the gradient sweep."""
-    n = 3 + (1 if n_groups * n_traj > 1 << 20 else 0)
+    statistics, with many groups the group statistics before them; GSPO adds
+    the per-trajectory pass and the gradient sweep."""
+    # GRPO whose trajectory tables fit 48 KB has an advantage kernel of its own
+    grpo_kernel = params.get("estimator", "grpo") == "grpo" and (4 * n_traj + 1) * 4 <= 48 * 1024
+    n = 3 + int(n_groups * n_traj > 1 << 20 if grpo_kernel else n_groups > 64)
     return n + (2 if params.get("estimator", "grpo") == "gspo" else 0)
 
 

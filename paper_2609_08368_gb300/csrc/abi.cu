@@ -542,15 +542,17 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
   // ends (eager calls of 2,048 x 4,096 23.1 -> 20 us); past that the waiting
   // CTAs are in the way as often as they help (3,488 x 43,648 with top-K 127.0
   // -> 132.0 us, two vocabulary shards of 4,096 rows 657 -> 645).
-  const bool early = overlap && c.R <= kEarlyStartRows;
-  aa.groups_done = group_kernel_pays(f.n_groups, f.n_traj);
+  bool grpo = aa.estimator == RL_EST_GRPO && aa.smem_traj && aa.n_traj > 0 && !aa.counts_out;
+  aa.groups_done = group_kernel_pays(grpo, f.n_groups, f.n_traj);
+  if (aa.groups_done) grpo = false;
+  // (k_groups in front makes it slower: 1,024 rows, 128 groups of 8, REINFORCE++
+  // 94 us started early, 59 not)
+  const bool early = overlap && c.R <= kEarlyStartRows && !aa.groups_done;
   if (aa.groups_done) {
     const int gb = std::min(f.n_groups, kMaxGroupBlocks);
     st = launch(groups_kernel(), dim3(static_cast<unsigned>(gb)), dim3(32), 0, 1, s, &aa, early);
     if (st != RL_OK) return st;
   }
-  const bool grpo = aa.estimator == RL_EST_GRPO && aa.smem_traj && !aa.groups_done &&
-                    aa.n_traj > 0 && !aa.counts_out;
   const void* fn = grpo ? adv_grpo_kernel() : adv_kernel();
   // tables and static shared memory together may pass the default 48 KB
   if (aa.smem_traj && traj_bytes > 48 * 1024 - static_cast<size_t>(kAdvStaticBytes)) {

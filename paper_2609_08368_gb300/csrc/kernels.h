@@ -283,11 +283,19 @@ inline int adv_grpo_ctas(long long rows, int n_traj) {
 }
 const void* groups_kernel();  // one 32-thread block per group (grid-stride)
 constexpr int kMaxGroupBlocks = 65535;
-// k_advantages computes the group statistics itself unless its cluster's
-// warps (128) would scan the trajectories for several hundred steps of 32
-// each: then k_groups spreads the groups over the whole GPU first.
-inline bool group_kernel_pays(long long n_groups, long long n_traj) {
-  return n_groups * n_traj > (1LL << 20);
+// Whether k_groups spreads the group statistics over the whole GPU before the
+// advantage kernel, which else forms them itself. k_advantages' 128 warps deal
+// the groups among them and queue for the SMs' double units: from some 64
+// groups on that is longer than another launch (REINFORCE++, 3,072 rows x 2,048,
+// inside / in k_groups, us: 64 groups of 16 62 / 64, 128 of 4 56 / 50, 128 of 8
+// 76 / 64, 256 of 4 105 / 64; 4,096 rows, 512 of 4 268 / 94; GRPO of 4,096
+// trajectories, 16 / 64 / 256 groups 157 / 179 / 326 against 168 / 172 / 179).
+// k_adv_grpo spreads the trajectories over up to 33 CTAs and forms a group in
+// every CTA that meets it, so groups times trajectories count: 128 x 1,024
+// 35 / 47, 256 x 1,024 37 / 47, 128 x 2,048 80 / 74, 512 x 2,048 86 / 77,
+// 1,024 x 2,048 125 / 81.
+inline bool group_kernel_pays(bool grpo_kernel, long long n_groups, long long n_traj) {
+  return grpo_kernel ? n_groups * n_traj > (1LL << 20) : n_groups > 64;
 }
 const void* seq_kernel();
 const void* merge_kernel();   // vocabulary-sharded calls: k_vmerge

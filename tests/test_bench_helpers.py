@@ -23,6 +23,10 @@ def test_launches_per_call():
     assert bench.launches_per_call({}, 1024, 1025) == 4  # past that k_groups
     assert bench.launches_per_call({"estimator": "gspo"}, 4, 64) == 5  # + k_seq, k_bwd
     assert bench.launches_per_call({"estimator": "reinforcepp"}, 1, 4) == 3
+    assert bench.launches_per_call({"estimator": "reinforcepp"}, 64, 512) == 3
+    assert bench.launches_per_call({"estimator": "reinforcepp"}, 65, 520) == 4  # more than 64 groups
+    assert bench.launches_per_call({}, 65, 3071) == 3
+    assert bench.launches_per_call({}, 65, 3072) == 4    # tables past 48 KB: k_advantages
 
 
 def test_sweep_kernel_name_follows_the_plan_tiers():

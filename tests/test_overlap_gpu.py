@@ -2,7 +2,9 @@
 dependents); recording events around the sweep makes the same call run them one
 after the other. No call may be slower for the overlap. The margin is far above
 what one box's timings differ by, and far below what a sweep loses that gets
-its places on the GPU in two rounds (20 to 40 %)."""
+its places on the GPU in two rounds (20 to 40 %).
+The same for the group statistics, which a kernel of their own forms where the
+advantage kernel would take longer."""
 
 import pytest
 import torch
@@ -59,3 +61,17 @@ def test_overlap_does_not_slow_a_call(vocab, rows, n_traj, estimator):
     finally:
         ml.rl_set_sweep_events()
     assert overlapped <= 1.08 * apart, f"{overlapped * 1e3:.1f} us against {apart * 1e3:.1f} one by one"
+
+
+@pytest.mark.parametrize("estimator,n_traj,few,many", [
+    ("reinforcepp_baseline", 2048, 64, 512), ("gspo", 2048, 64, 512), ("grpo", 4096, 16, 256)])
+def test_many_groups_cost_little_more_than_few(estimator, n_traj, few, many):
+    times = []
+    for n_groups in (few, many):
+        rec = wl.shrink(wl.RECIPES["glm"], n_prompts=n_groups, group_size=n_traj // n_groups,
+                        traj_len=2, vocab=2048)
+        w = wl.make(rec, DEV)
+        params = dict(w.params, estimator=estimator)
+        buf = api.alloc(w.n_rows, n_traj, n_groups, DEV, vocab=2048, dlogits_dtype=w.logits.dtype)
+        times.append(_fastest(lambda: api.fwd_bwd(w, buf, params=params)))
+    assert times[1] <= 1.5 * times[0], [f"{t * 1e3:.1f} us" for t in times]
