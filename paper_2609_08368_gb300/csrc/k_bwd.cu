@@ -140,11 +140,23 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd(const BwdArgs a) {
       }
       Out::template storev<V8>(drow + static_cast<size_t>(jb) * Out::kSize, f, 0u);
     }
-    const int before = kUnal ? min(jv, j1) - j0 : 0;
+    // the elements that no vector holds
     const int skip = nv * V8;
-    for (int e = threadIdx.x; e < j1 - j0 - skip; e += kBwdThreads) {
-      const int j = j0 + e + (e >= before ? skip : 0);
+    auto element = [&](int j) {
       Out::store1(drow, j, cc == 0.0f ? 0.0f : value(In::load1(zrow, j), j));
+    };
+    if constexpr (kUnal) {
+      if (head < 0) {
+        // (a loop of its own, which the compiler can unroll: 4,096 rows x 16,632
+        // bf16 376 -> 209 us, x 45,003 727 -> 560)
+        for (int j = j0 + skip + threadIdx.x; j < j1; j += kBwdThreads) element(j);
+      } else {
+        const int before = min(jv, j1) - j0;
+        for (int e = threadIdx.x; e < j1 - j0 - skip; e += kBwdThreads)
+          element(j0 + e + (e >= before ? skip : 0));
+      }
+    } else {
+      for (int e = threadIdx.x; e < j1 - j0 - skip; e += kBwdThreads) element(j0 + e + skip);
     }
 #pragma unroll
     for (int i = 0; i < kPer; ++i) raw[i] = nxt[i];
