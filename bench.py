@@ -289,8 +289,9 @@ def sweep_kernel_label(vocab: int, elem_size: int, grad: bool = True, topk: bool
     """sweep_kernel_name, and what it leaves out: with nothing forced, the
     short-row kernel for rows below 20 KB, and for rows that do not all start
     on a 16-byte boundary (in the logits and in dLogits alike: not
-    ``aligned``) the streaming kernel's unaligned forms: bf16 rows of any
-    length, fp32 rows from 4 KB on in the cluster kernel's slices."""
+    ``aligned``) the streaming kernel's unaligned forms, past the shortest
+    rows: bf16 from 1.5 KB (forward only 1.25, with top-K 5), fp32, in the
+    cluster kernel's slices, from 8 KB."""
     KB, row_bytes = 1024, vocab * elem_size
     kind = "fused fwd+bwd" if grad else "forward-only"
     if aligned and row_bytes < 20 * KB and not forced and not forced_cluster:
@@ -298,9 +299,11 @@ def sweep_kernel_label(vocab: int, elem_size: int, grad: bool = True, topk: bool
     if aligned or forced == "cluster":
         return sweep_kernel_name(vocab, elem_size, grad, topk, forced, forced_cluster)
     if elem_size == 4:
-        if forced or forced_cluster or row_bytes < 4 * KB:
+        if forced or forced_cluster or row_bytes < 8 * KB:
             return sweep_kernel_name(vocab, elem_size, grad, topk, forced="cluster")
         return f"k_stream ({kind} vocabulary sweep, unaligned rows, one CTA per row, 2 CTAs per SM)"
+    if not forced and row_bytes < (5 * KB if topk else (1536 if grad else 1280)):
+        return sweep_kernel_name(vocab, elem_size, grad, topk, forced="cluster")
     # bf16: the tiers of aligned rows; where those have the cluster kernel, CTAs
     # per SM by length
     name = sweep_kernel_name(vocab, elem_size, grad, topk, forced_cluster=forced_cluster)

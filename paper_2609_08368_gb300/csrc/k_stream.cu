@@ -12,6 +12,7 @@ bool use_stream(long long row_bytes, int es, bool in_bulk, bool unal, bool grad,
   // a launch shape forced, and below kVirtRowBytes, by that kernel itself)
   if (es == 4 && !in_bulk) return !plan_forced(ov) && row_bytes >= kVirtRowBytes;
   if (ov.sweep_kernel == 1) return true;
+  if (es == 2 && unal && row_bytes < unal_stream_bytes(in_bulk, grad, topk)) return false;
   return stream_ctas(row_bytes, es, grad, topk, unal && es == 2) > 0;
 }
 

@@ -63,8 +63,9 @@ inline bool halves_row(long long row_bytes, int es, bool grad, bool unal) {
 
 // unal: bf16 rows that do not all start on a 16-byte boundary. The cluster
 // kernel reads and writes those element by element (4,096 x 45,003: 937 us
-// against 135), so every length streams: those the table above gives to the
-// cluster kernel with the CTAs per SM that came closest to it there.
+// against 135), so all but the shortest (unal_stream_bytes) stream: those the
+// table above gives to the cluster kernel with the CTAs per SM that came
+// closest to it there.
 inline int stream_ctas(long long row_bytes, int es, bool grad, bool topk, bool unal = false) {
   constexpr long long KB = 1024;
   if (unal) {
@@ -102,9 +103,23 @@ inline bool plan_forced(const rl_launch_overrides& ov) {
 inline bool use_short(long long row_bytes, bool unal, const rl_launch_overrides& ov) {
   return !plan_forced(ov) && !unal && row_bytes < kShortRowBytes;
 }
-// Unaligned fp32 rows from this length on: k_stream in the cluster kernel's
-// order (4,096 rows of 4 KB: 57 us a call against 61, of 9 KB 59 against 92).
-constexpr long long kVirtRowBytes = 4 * 1024;
+// Unaligned rows stream from these lengths on; shorter ones take the cluster
+// kernel, element by element (streamed / that kernel, us a call; 16,384 rows,
+// or 1,024 where said). fp32, in the cluster kernel's order: 4 KB 178 / 128, 6
+// KB 184 / 163, 8 KB 186 / 198 (1,024: 22.3 / 21.8), 12 KB 189 / 272.
+constexpr long long kVirtRowBytes = 8 * 1024;
+// bf16: fused 0.4 KB 105 / 81, 1.5 KB 112 / 107 (1,024: 17.7 / 18.8), 3 KB 115 /
+// 127; forward only 0.6 KB 71 / 68, 1 KB 73 / 69, 1.5 KB 73 / 83; with top-K, whose
+// warp waits for every row's copy, 1 KB 202 / 107, 4 KB 212 / 191, 6 KB 220 / 259
+// (1,024: 4 KB 24.3 / 22.9, 6 KB 24.7 / 24.8). Where only dLogits are unaligned the
+// cluster kernel still copies its rows whole: 2 KB 102 / 94, 3 KB 106 / 101 (1,024:
+// 17.1 / 18.4), 4 KB 108 / 109; with top-K 12 KB 227 / 190, 16 KB 235 / 222 (6,144
+// rows: 97 / 103).
+inline long long unal_stream_bytes(bool in_bulk, bool grad, bool topk) {
+  if (in_bulk) return topk ? 16 * 1024 : 3 * 1024;
+  if (topk) return 5 * 1024;
+  return grad ? 1536 : 1280;
+}
 // Warps per row and vectors per lane that hold a row of n_vec vectors.
 inline void short_shape(long long n_vec, int* warps, int* nv) {
   *warps = n_vec <= 512 ? 1 : (n_vec <= 1024 ? 2 : 4);

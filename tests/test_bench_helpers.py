@@ -88,7 +88,9 @@ def test_sweep_kernel_label():
     assert label(4096, 2, forced="cluster").startswith("k_sweep")
     assert label(154880, 2) == bench.sweep_kernel_name(154880, 2)
     unal, un = "k_stream (fused fwd+bwd vocabulary sweep, unaligned rows", dict(aligned=False)
-    assert label(1001, 2, **un) == unal + ", one CTA per row, 4 CTAs per SM)"
+    assert label(1025, 2, **un) == unal + ", one CTA per row, 4 CTAs per SM)"
+    assert label(767, 2, **un).startswith("k_sweep")                        # below 1.5 KB
+    assert label(2001, 2, topk=True, **un).startswith("k_sweep")            # below 5 KB
     assert label(45003, 2, **un) == unal + ", one CTA per row, 2 CTAs per SM)"  # 88 KB
     assert label(75003, 2, **un) == unal + ", one CTA per row)"             # 146 KB
     assert label(154883, 2, **un) == unal + ", one CTA per row)"
@@ -96,9 +98,9 @@ def test_sweep_kernel_label():
     assert label(8001, 2, topk=True, **un) == unal + ", one CTA per row, 2 CTAs per SM)"
     assert label(45003, 2, forced="cluster", **un).startswith("k_sweep")
     assert label(45003, 2, forced="stream", **un) == label(45003, 2, **un)
-    # fp32: the cluster kernel's slices, from 4 KB on and with nothing forced
+    # fp32: the cluster kernel's slices, from 8 KB on and with nothing forced
     assert label(32769, 4, **un) == unal + ", one CTA per row, 2 CTAs per SM)"
-    assert label(1001, 4, **un).startswith("k_sweep")
+    assert label(2047, 4, **un).startswith("k_sweep")
     assert label(32769, 4, forced="stream", **un).startswith("k_sweep")
 
 

@@ -7,6 +7,7 @@ import pytest
 import torch
 
 from paper_2609_08368_gb300 import api
+from paper_2609_08368_gb300 import milesloss as ml
 from paper_2609_08368_gb300 import workloads as wl
 
 pytestmark = pytest.mark.gpu
@@ -56,3 +57,19 @@ def test_gradient_of_rows_misaligned_against_each_other(dtype):
         api.fwd(w, buf)
         times.append(_fastest(lambda: api.bwd(w, buf)))
     assert times[1] <= 5.2 * times[0], times
+
+
+@pytest.mark.parametrize("dtype,vocab,off,topk,mode", [
+    ("bf16", 201, 1, 0, "fused"), ("bf16", 201, 1, 8, "fused"), ("bf16", 511, 1, 8, "fwd"),
+    ("bf16", 1537, 1, 0, "fused"), ("bf16", 3001, 1, 8, "fused"), ("bf16", 1025, 1, 0, "fwd"),
+    ("bf16", 320, 0, 0, "fused"), ("bf16", 2048, 0, 8, "fused"), ("bf16", 3072, 0, 0, "fused"),
+    ("f32", 1025, 1, 0, "fused"), ("f32", 1025, 1, 0, "fwd"), ("f32", 3001, 1, 8, "fused")])
+def test_short_unaligned_rows_take_the_faster_kernel(dtype, vocab, off, topk, mode):
+    """Logits that start `off` elements past a boundary, dLogits that do too
+    (or, where the logits are aligned, two elements past one)."""
+    w, buf = _batch(dtype, 16384, vocab, off, off or 2, topk)
+    call = (lambda: api.fwd_bwd(w, buf)) if mode == "fused" else (lambda: api.fwd(w, buf))
+    chosen = _fastest(call)
+    with ml.launch_overrides(sweep_kernel="cluster"):
+        other = _fastest(call)
+    assert chosen <= 1.06 * other, (chosen, other)
