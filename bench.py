@@ -283,30 +283,31 @@ def sweep_kernel_name(vocab: int, elem_size: int, grad: bool = True, topk: bool 
     return f"k_sweep ({kind} vocabulary sweep, clusters sharing a row)"
 
 
-def sweep_kernel_label(vocab: int, elem_size: int, grad: bool = True, topk: bool = False,
+def sweep_kernel_label(vocab: int, elem_size: int, grad: bool = True, topk: int = 0,
                        forced: str | None = None, forced_cluster: int | None = None,
                        aligned: bool = True) -> str:
     """sweep_kernel_name, and what it leaves out: with nothing forced, the
-    short-row kernel for rows below 20 KB, and for rows that do not all start
-    on a 16-byte boundary (in the logits and in dLogits alike: not
-    ``aligned``) the streaming kernel's unaligned forms, past the shortest
-    rows: bf16 from 1.5 KB (forward only 1.25, with top-K 5), fp32, in the
-    cluster kernel's slices, from 8 KB."""
+    short-row kernel for rows below 20 KB (up to 16 with top-K past K = 32;
+    ``topk`` is K), and for rows that do not all start on a 16-byte boundary
+    (in the logits and in dLogits alike: not ``aligned``) the streaming
+    kernel's unaligned forms, past the shortest rows: bf16 from 1.5 KB (forward
+    only 1.25, with top-K 5), fp32, in the cluster kernel's slices, from 8 KB."""
     KB, row_bytes = 1024, vocab * elem_size
     kind = "fused fwd+bwd" if grad else "forward-only"
-    if aligned and row_bytes < 20 * KB and not forced and not forced_cluster:
+    short = row_bytes < 20 * KB and (topk <= 32 or row_bytes <= 16 * KB)
+    if aligned and short and not forced and not forced_cluster:
         return f"k_short ({kind} vocabulary sweep, a row in the registers of one to four warps)"
     if aligned or forced == "cluster":
-        return sweep_kernel_name(vocab, elem_size, grad, topk, forced, forced_cluster)
+        return sweep_kernel_name(vocab, elem_size, grad, bool(topk), forced, forced_cluster)
     if elem_size == 4:
         if forced or forced_cluster or row_bytes < 8 * KB:
-            return sweep_kernel_name(vocab, elem_size, grad, topk, forced="cluster")
+            return sweep_kernel_name(vocab, elem_size, grad, bool(topk), forced="cluster")
         return f"k_stream ({kind} vocabulary sweep, unaligned rows, one CTA per row, 2 CTAs per SM)"
     if not forced and row_bytes < (5 * KB if topk else (1536 if grad else 1280)):
-        return sweep_kernel_name(vocab, elem_size, grad, topk, forced="cluster")
+        return sweep_kernel_name(vocab, elem_size, grad, bool(topk), forced="cluster")
     # bf16: the tiers of aligned rows; where those have the cluster kernel, CTAs
     # per SM by length
-    name = sweep_kernel_name(vocab, elem_size, grad, topk, forced_cluster=forced_cluster)
+    name = sweep_kernel_name(vocab, elem_size, grad, bool(topk), forced_cluster=forced_cluster)
     if name.startswith("k_sweep"):
         per = 1 if grad and row_bytes >= 136 * KB else (2 if topk or row_bytes > 56 * KB else 4)
         name = f"k_stream ({kind} vocabulary sweep, one CTA per row" + \
@@ -833,7 +834,7 @@ def run_ours(args, rank, world, local):
     bpr = algorithmic_bytes_per_row(w, dl_dtype)  # before w is released for the e2e leg
     aligned = all(t.data_ptr() % 16 == 0 and t.stride(0) * t.element_size() % 16 == 0
                   for t in (w.logits, buf.dlogits))
-    kernel_name = sweep_kernel_label(V, w.logits.element_size(), topk=bool(args.opd_topk),
+    kernel_name = sweep_kernel_label(V, w.logits.element_size(), topk=args.opd_topk,
                                     forced=args.sweep_kernel, forced_cluster=args.stream_cluster,
                                     aligned=aligned)
     w_params, n_groups, n_traj = dict(w.params), w.n_groups, int(w.rewards.shape[0])
@@ -844,7 +845,7 @@ def run_ours(args, rank, world, local):
         # sweep k_bwd follow it): it reads the logits and writes no dLogits
         launch_bytes = (bpr - V * torch.tensor([], dtype=dl_dtype).element_size()) * R
         kernel_name = sweep_kernel_label(V, w.logits.element_size(), grad=False,
-                                        topk=bool(args.opd_topk), forced=args.sweep_kernel,
+                                        topk=args.opd_topk, forced=args.sweep_kernel,
                                         aligned=aligned) + \
             ", GSPO's first pass (k_bwd reads the logits again for dLogits)"
     sweep_avg = statistics.fmean(sweep_ms)

@@ -619,7 +619,7 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     if (st == RL_ERR_UNSUPPORTED) stream = false;
     else if (st != RL_OK) return st;
   }
-  if (c.R > 0 && use_short(row_bytes, unal, ov)) {
+  if (c.R > 0 && use_short(row_bytes, unal, sc.topk, ov)) {
     int warps = 0, nv = 0, sms = 0;
     short_shape(row_bytes / 16, &warps, &nv);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)

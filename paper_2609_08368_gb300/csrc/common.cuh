@@ -700,9 +700,10 @@ __device__ __forceinline__ TopKPart topk_merge_all(const float4* parts, int n) {
 }
 
 // The warp's part over its lanes' candidates whose ids satisfy `mine`
-// (fixed-order butterfly; every lane ends with it); k = log2(e) / T.
-template <class Mine>
-__device__ __forceinline__ TopKPart topk_part(const TopKLane& c, const float* teacher, int lane,
+// (fixed-order butterfly; every lane ends with it); k = log2(e) / T, teacher(i)
+// the teacher's log-prob of candidate i (the lane's own, lane or lane + 32).
+template <class Teacher, class Mine>
+__device__ __forceinline__ TopKPart topk_part(const TopKLane& c, Teacher teacher, int lane,
                                               float invT, float k, Mine mine) {
   const bool u0 = c.id0 >= 0 && mine(c.id0), u1 = c.id1 >= 0 && mine(c.id1);
   const int bad = __any_sync(0xffffffffu, c.bad) ? 1 : 0;
@@ -713,8 +714,8 @@ __device__ __forceinline__ TopKPart topk_part(const TopKLane& c, const float* te
   if (M == -INFINITY) return TopKPart{-INFINITY, 0.0f, 0.0f, bad};
   const float w0 = u0 ? ex2(t0 - M) : 0.0f, w1 = u1 ? ex2(t1 - M) : 0.0f;
   float sw = w0 + w1;
-  float acc = (u0 ? w0 * fmaf(c.z0, invT, -teacher[lane]) : 0.0f) +
-              (u1 ? w1 * fmaf(c.z1, invT, -teacher[lane + 32]) : 0.0f);
+  float acc = (u0 ? w0 * fmaf(c.z0, invT, -teacher(lane)) : 0.0f) +
+              (u1 ? w1 * fmaf(c.z1, invT, -teacher(lane + 32)) : 0.0f);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     sw += __shfl_xor_sync(0xffffffffu, sw, o);

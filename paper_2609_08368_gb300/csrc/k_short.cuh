@@ -120,12 +120,21 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
 
   // ---------------- loads: the row, its scalars
   // top-K OPD: the row's candidates in these columns (the group's first
-  // warp): the ids first, their logits once the row is on its way, the part
-  // after pass A
+  // warp): the ids and the teacher's values first, their logits once the row is
+  // on its way, the part after pass A. (The values behind pass A, where they
+  // are used, cost a load's latency a row: 65,536 rows x 2,048 / 4,096 fp32, K =
+  // 32, 216 / 397 -> 198 / 363 us. With sixteen vectors of bf16 a lane there are no
+  // registers for them: x 4,096 261 us early, 252 late.)
+  constexpr bool kTeachEarly = !(kW == 1 && kNV > 8 && V8 == 8);
   TopKLane tk{-1, -1, 0.0f, 0.0f, false};
-  if (kTopK && w == 0)
+  float teach0 = 0.0f, teach1 = 0.0f;
+  const float* teacher = a.s.topk_teacher + (kTopK ? row * a.s.topk : 0);
+  if (kTopK && w == 0) {
+    if (kTeachEarly && lane < a.s.topk) teach0 = teacher[lane];
+    if (kTeachEarly && lane + 32 < a.s.topk) teach1 = teacher[lane + 32];
     tk = topk_ids(a.s.topk_ids + row * a.s.topk, static_cast<int>(a.col0), a.V, a.vocab_total,
                   a.s.topk, lane);
+  }
   uint4 raw[kNV];
 #pragma unroll
   for (int i = 0; i < kNV; ++i)
@@ -265,8 +274,8 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
   }
   TopKPart part{-INFINITY, 0.0f, 0.0f, 0};
   if (kTopK && w == 0) {
-    part = topk_part(tk, a.s.topk_teacher + row * a.s.topk, lane, a.s.invT, k,
-                     [](int) { return true; });
+    auto value = [=](int i) { return kTeachEarly ? (i < 32 ? teach0 : teach1) : teacher[i]; };
+    part = topk_part(tk, value, lane, a.s.invT, k, [](int) { return true; });
     if (lane == 0) tkp[grp] = part;
   }
   if (kW > 1) asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(kT) : "memory");

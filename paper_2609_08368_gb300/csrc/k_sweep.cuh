@@ -340,7 +340,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep(const SweepArgs 
       if (have) topk_gather<In>(tk, sb, lo, lo + vec_elems);
       topk_gather<In>(tk, grow + static_cast<size_t>(vec_elems) * sizeof(St), lo + vec_elems, lo + cnt);
       const int c0 = lo, c1 = lo + cnt;
-      tkp = topk_part(tk, tk_row->teacher, tid, a.s.invT, k, [c0, c1](int id) { return id >= c0 && id < c1; });
+      tkp = topk_part(tk, [=](int i) { return tk_row->teacher[i]; }, tid, a.s.invT, k,
+                      [c0, c1](int id) { return id >= c0 && id < c1; });
     }
     if (it == 0 && tid == 0) {
       // the advantage kernel's results: it may still be running until here

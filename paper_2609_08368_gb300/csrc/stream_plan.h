@@ -90,8 +90,14 @@ inline int stream_ctas(long long row_bytes, int es, bool grad, bool topk, bool u
 
 // Rows of up to kShortRowBytes that start 16-byte aligned (logits and
 // dLogits): k_short, with the row in registers, unless an override asks for a
-// launch shape of the other kernels.
+// launch shape of the other kernels. With top-K OPD (topk = K) one of a row's
+// four warps has the candidates while the others wait: past 16 KB and K = 32
+// the cluster kernel is faster (k_short / k_sweep, us, 18 KB rows, K = 64: bf16
+// fused 16,384 rows 153 / 142, 65,536 577 / 530, forward only 65,536 395 / 380, fp32
+// fused 65,536 512 / 476; but 1,024 rows 18.4 / 19.8. K = 32: bf16 fused 4,096 44 /
+// 46, 16,384 146 / 140, 65,536 552 / 519, forward only 325 / 372, fp32 fused 435 / 461).
 constexpr long long kShortRowBytes = 20 * 1024;
+constexpr long long kShortTopKBytes = 16 * 1024;
 inline bool plan_forced(const rl_launch_overrides& ov) {
   return ov.sweep_kernel >= 0 || ov.cluster_size > 0 || ov.cluster_stages > 0 ||
          ov.cluster_threads > 0 || ov.cluster_ctas_per_sm > 0 ||
@@ -100,7 +106,8 @@ inline bool plan_forced(const rl_launch_overrides& ov) {
          ov.stream_ctas_per_sm > 0 || ov.stream_cluster > 0 ||
          ov.stall_first_wait_ns > 0;
 }
-inline bool use_short(long long row_bytes, bool unal, const rl_launch_overrides& ov) {
+inline bool use_short(long long row_bytes, bool unal, int topk, const rl_launch_overrides& ov) {
+  if (topk > 32 && row_bytes > kShortTopKBytes) return false;
   return !plan_forced(ov) && !unal && row_bytes < kShortRowBytes;
 }
 // Unaligned rows stream from these lengths on; shorter ones take the cluster

@@ -86,16 +86,19 @@ def test_sweep_kernel_label():
     assert label(10232, 2, grad=False).startswith("k_short (forward-only")
     assert label(10240, 2) == bench.sweep_kernel_name(10240, 2)            # 20 KB
     assert label(4096, 2, forced="cluster").startswith("k_sweep")
+    assert label(8192, 2, topk=64).startswith("k_short")                    # 16 KB
+    assert label(8200, 2, topk=33).startswith("k_sweep")
+    assert label(8200, 2, topk=32).startswith("k_short")
     assert label(154880, 2) == bench.sweep_kernel_name(154880, 2)
     unal, un = "k_stream (fused fwd+bwd vocabulary sweep, unaligned rows", dict(aligned=False)
     assert label(1025, 2, **un) == unal + ", one CTA per row, 4 CTAs per SM)"
     assert label(767, 2, **un).startswith("k_sweep")                        # below 1.5 KB
-    assert label(2001, 2, topk=True, **un).startswith("k_sweep")            # below 5 KB
+    assert label(2001, 2, topk=8, **un).startswith("k_sweep")            # below 5 KB
     assert label(45003, 2, **un) == unal + ", one CTA per row, 2 CTAs per SM)"  # 88 KB
     assert label(75003, 2, **un) == unal + ", one CTA per row)"             # 146 KB
     assert label(154883, 2, **un) == unal + ", one CTA per row)"
     assert label(250001, 2, **un) == unal + ", a cluster of 2 CTAs per row)"
-    assert label(8001, 2, topk=True, **un) == unal + ", one CTA per row, 2 CTAs per SM)"
+    assert label(8001, 2, topk=8, **un) == unal + ", one CTA per row, 2 CTAs per SM)"
     assert label(45003, 2, forced="cluster", **un).startswith("k_sweep")
     assert label(45003, 2, forced="stream", **un) == label(45003, 2, **un)
     # fp32: the cluster kernel's slices, from 8 KB on and with nothing forced

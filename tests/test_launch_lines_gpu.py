@@ -73,3 +73,16 @@ def test_short_unaligned_rows_take_the_faster_kernel(dtype, vocab, off, topk, mo
     with ml.launch_overrides(sweep_kernel="cluster"):
         other = _fastest(call)
     assert chosen <= 1.06 * other, (chosen, other)
+
+
+@pytest.mark.parametrize("dtype,vocab,topk,mode", [
+    ("bf16", 8192, 64, "fused"), ("bf16", 9216, 16, "fused"), ("bf16", 9216, 64, "fused"),
+    ("bf16", 9216, 32, "fwd"), ("bf16", 9216, 64, "fwd"), ("f32", 4608, 32, "fused"),
+    ("f32", 4608, 64, "fused")])
+def test_short_rows_with_topk_take_the_faster_kernel(dtype, vocab, topk, mode):
+    w, buf = _batch(dtype, 16384, vocab, 0, 0, topk)
+    call = (lambda: api.fwd_bwd(w, buf)) if mode == "fused" else (lambda: api.fwd(w, buf))
+    chosen = _fastest(call)
+    with ml.launch_overrides(sweep_kernel="cluster"):
+        other = _fastest(call)
+    assert chosen <= 1.06 * other, (chosen, other)
