@@ -714,8 +714,9 @@ __device__ __forceinline__ TopKPart topk_part(const TopKLane& c, Teacher teacher
   if (M == -INFINITY) return TopKPart{-INFINITY, 0.0f, 0.0f, bad};
   const float w0 = u0 ? ex2(t0 - M) : 0.0f, w1 = u1 ? ex2(t1 - M) : 0.0f;
   float sw = w0 + w1;
-  float acc = (u0 ? w0 * fmaf(c.z0, invT, -teacher(lane)) : 0.0f) +
-              (u1 ? w1 * fmaf(c.z1, invT, -teacher(lane + 32)) : 0.0f);
+  // (a candidate of probability zero adds nothing, also where its logit is -inf)
+  float acc = (w0 != 0.0f ? w0 * fmaf(c.z0, invT, -teacher(lane)) : 0.0f) +
+              (w1 != 0.0f ? w1 * fmaf(c.z1, invT, -teacher(lane + 32)) : 0.0f);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     sw += __shfl_xor_sync(0xffffffffu, sw, o);

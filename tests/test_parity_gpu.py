@@ -647,6 +647,32 @@ def test_a_forward_only_wait_that_runs_out_is_reported(ov, name, vocab, topk, st
     _full_check(w, mode="fwd", params=params)
 
 
+@pytest.mark.parametrize("name,vocab", [
+    ("glm", 4096), ("glm", 32768), ("glm", 45056), ("glm", 110000), ("glm", 3001), ("glm", 45003),
+    ("fp32", 4096), ("fp32", 65792), ("fp32", 10001)])
+@pytest.mark.parametrize("mode", ["fused", "fwd"])
+def test_topk_candidate_of_probability_zero(name, vocab, mode):
+    """A candidate whose logit is -inf has weight 0 in the signal, in every
+    sweep kernel, whichever part of the row its column is in. (The oracle is
+    given -5,000 in its place: a weight of exactly 0 there, a finite log-prob.)"""
+    rec = wl.shrink(wl.RECIPES[name], n_prompts=1, group_size=2, traj_len=3, vocab=vocab, topk=8,
+                    rho_noise=0.3, mask="none")
+    w = wl.make(rec, DEV)
+    w.logits[1, vocab // 3:2 * vocab // 3] = -float("inf")
+    w.logits[4, :vocab // 3] = -float("inf")
+    w.targets[1], w.targets[4] = 5, vocab - 5
+    w.topk_ids[1, 2], w.topk_ids[1, 7] = vocab // 2, 1
+    w.topk_ids[4, 0], w.topk_ids[4, 1] = 0, vocab - 2
+    params = dict(w.params, opd_topk=8, opd_coef=0.5)
+    g = P.run_gpu(w, mode=mode, params=params)
+    assert g["err"] == 0
+    w.logits.clamp_(min=-5000.0)
+    o = P.run_oracle(w, params=params)
+    P.assert_loss_close(g["stats"]["loss"], o["stats"]["loss"])
+    if mode == "fused":
+        P.assert_dlogits_close(g["dlogits_t"].float().cpu().numpy(), o["dlogits"])
+
+
 @pytest.mark.parametrize("kind,cluster", [("cluster", 0), ("cluster", 4), ("stream", 0)])
 def test_topk_ids_out_of_range_are_reported(ov, kind, cluster):
     """A top-K OPD candidate id outside [0, vocab) zeros its row (as a bad
