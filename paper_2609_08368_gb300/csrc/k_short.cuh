@@ -41,36 +41,6 @@ namespace {
 
 constexpr float kLn2s = 0.69314718055994531f;
 
-// Logits below this have probability zero whatever the rest of the row: pass A
-// takes them (and -inf) as this, so that p (z k - m) is -0 and not NaN.
-constexpr float kShortFloor = -1.0e30f;
-
-// max(w, kShortFloor) of every element, NaN kept.
-struct FloorBf16 {
-  static __device__ __forceinline__ uint4 apply(uint4 w) {
-    constexpr uint32_t f2 = 0xf149f149u;  // bf16 -9.95e29, twice
-    auto m = [](uint32_t x) {
-      uint32_t r;
-      asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(f2));
-      return r;
-    };
-    return make_uint4(m(w.x), m(w.y), m(w.z), m(w.w));
-  }
-};
-struct FloorF32 {
-  static __device__ __forceinline__ uint4 apply(uint4 w) {
-    auto m = [](uint32_t x) {
-      float r;
-      asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(__uint_as_float(x)), "f"(kShortFloor));
-      return __float_as_uint(r);
-    };
-    return make_uint4(m(w.x), m(w.y), m(w.z), m(w.w));
-  }
-};
-template <class In> struct FloorOf;
-template <> struct FloorOf<InBf16> : FloorBf16 {};
-template <> struct FloorOf<InF32> : FloorF32 {};
-
 // The warp's maximum (fp32 order by an order-preserving map to integers).
 __device__ __forceinline__ float warp_max_redux(float v) {
   const int i = __float_as_int(v);
@@ -169,8 +139,7 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
   const float k = a.s.k;
   const float2 k2 = make_float2(k, k);
   float vm[kJ], vs[kJ], vu[kJ];
-  // against the reference r; safe: logits far below any that matter taken at
-  // the floor (the usual sums skip that)
+  // against the reference r; safe: with floor_t (the usual sums skip that)
   auto sums = [&](auto safe, int j, float r, float& s, float& u) {
     const float2 nr2 = make_float2(-r, -r);
     float2 s0 = make_float2(0.0f, 0.0f), s1 = s0, u0 = s0, u1 = s0;
@@ -179,10 +148,12 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
       const int i = j + kJ * ii;
       if (i < kNV && i * kT + t < n_vec) {
         float2 f[P];
-        In::unpack2(decltype(safe)::value ? FloorOf<In>::apply(raw[i]) : raw[i], f);
+        In::unpack2(raw[i], f);
 #pragma unroll
         for (int e = 0; e < P; ++e) {
-          const float2 x2 = ffma2(f[e], k2, nr2), x = ex2x2(x2);
+          float2 x2 = ffma2(f[e], k2, nr2);
+          if (decltype(safe)::value) x2 = floor_t2(x2);
+          const float2 x = ex2x2(x2);
           if (ii & 1) {
             s1 = fadd2(s1, x);
             u1 = ffma2(x, x2, u1);
@@ -206,10 +177,10 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
       const float r = In::vmax(raw[j]) * k;
       sums(std::false_type{}, j, r, vs[j], vu[j]);
       vm[j] = r;
-      if (!(fabsf(vs[j]) < INFINITY) || !(fabsf(vu[j]) < INFINITY) || r == -INFINITY) redo |= 1u << j;
+      if (!(fabsf(vs[j]) < INFINITY) || !(fabsf(vu[j]) < INFINITY) || r < kNoLogit) redo |= 1u << j;
     }
   }
-  if (redo) {  // (rare: an overflow, or a -inf logit) the thread's own maximum
+  if (redo) {  // (rare: an overflow, or a masked logit) the thread's own maximum
 #pragma unroll
     for (int j = 0; j < kJ; ++j) {
       if (!(redo >> j & 1u)) continue;
@@ -221,7 +192,8 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
       }
       vm[j] = In::max_val(macc) * k;
       vs[j] = vu[j] = 0.0f;
-      if (vm[j] != -INFINITY) sums(std::true_type{}, j, vm[j], vs[j], vu[j]);
+      if (vm[j] < kNoLogit) vm[j] = -INFINITY;
+      else sums(std::true_type{}, j, vm[j], vs[j], vu[j]);
     }
   }
   float most = vs[0];
@@ -239,8 +211,8 @@ __global__ void __launch_bounds__(kShortThreads, kNV > 10 ? 4 : 5) k_short(const
       }
     }
   }
-  if (has_tail && z_tail != -INFINITY) {  // (the block's first threads: j = 0 of warp 0)
-    const float zk = z_tail * k;
+  const float zk = z_tail * k;
+  if (has_tail && !(zk < kNoLogit)) {  // (the block's first threads: j = 0 of warp 0)
     if (zk > vm[0]) {
       if (vs[0] > 0.0f) {
         const float d = vm[0] - zk, f = ex2(d);

@@ -154,7 +154,7 @@ struct Run {
 
   // move the reference up to nr (sums rescaled by 2^(r - nr))
   __device__ __forceinline__ void raise(float nr) {
-    if (!(nr > r)) return;
+    if (!(nr > r) || nr < kNoLogit) return;
     if (r != -INFINITY) {
       const float d = r - nr, f = ex2(d);
       const float2 f2 = make_float2(f, f), d2 = make_float2(d, d);
@@ -183,10 +183,7 @@ struct Run {
   template <bool kSafe>
   __device__ __forceinline__ void add_pair(float2 z, float2 k2, float2& s, float2& u) {
     float2 t = ffma2(z, k2, make_float2(-r, -r));
-    if (kSafe) {
-      if (z.x == -INFINITY) t.x = -127.0f;
-      if (z.y == -INFINITY) t.y = -127.0f;
-    }
+    if (kSafe) t = floor_t2(t);
     const float2 x = ex2x2(t);
     s = fadd2(s, x);
     u = ffma2(x, t, u);
@@ -744,14 +741,14 @@ __global__ void __launch_bounds__(stream_threads(kTopK, kCW, kDec), 16 / kCW) k_
     // reference (for the first chunk, the maximum of the thread's first
     // vector): the sums are finite unless a logit lies more than 127 / k
     // above the reference, and that case (an overflow, seen as inf) or a
-    // -inf logit (NaN) redoes the chunk against the chunk's own maximum,
-    // skipping -inf logits exactly.
+    // masked logit (NaN) redoes the chunk against the chunk's own maximum,
+    // skipping masked logits exactly.
     Run run;
     Tri t{-INFINITY, 0.0f, 0.0f};
     // (kVirt, and the elements past the last whole vector)
     auto add1 = [&](float z) {
-      if (z == -INFINITY) return;
       const float zk = z * k;
+      if (zk < kNoLogit) return;
       if (zk > t.m) {
         if (t.s > 0.0f) {
           const float d = t.m - zk, f = ex2(d);

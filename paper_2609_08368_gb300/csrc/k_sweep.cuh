@@ -86,9 +86,9 @@ __device__ __forceinline__ Tri block_merge(Tri t, float4* red) {
 }
 
 // Sum of 2^(t - mt) and of 2^(t - mt) (t - mt) over the thread's vectors,
-// t = z k, for a fixed reference mt in log2 units. kSafe skips
-// -inf logits exactly (0 * -inf would otherwise give NaN); it runs only
-// when the fast pass produced a NaN.
+// t = z k, for a fixed reference mt in log2 units. kSafe skips masked
+// logits exactly (floor_t); it runs only when the fast pass produced a NaN or
+// an overflow.
 template <class In, int kThreads, bool kSafe>
 __device__ __forceinline__ void sum_pass(const uint4* sv, int n_vec, float k, float mt,
                                          float& s_out, float& u_out) {
@@ -105,10 +105,8 @@ __device__ __forceinline__ void sum_pass(const uint4* sv, int n_vec, float k, fl
     for (int e = 0; e < P; ++e) {
       float2 ta = ffma2(fa[e], k2, nm2), tb = ffma2(fb[e], k2, nm2);
       if (kSafe) {
-        if (fa[e].x == -INFINITY) ta.x = -127.0f;
-        if (fa[e].y == -INFINITY) ta.y = -127.0f;
-        if (fb[e].x == -INFINITY) tb.x = -127.0f;
-        if (fb[e].y == -INFINITY) tb.y = -127.0f;
+        ta = floor_t2(ta);
+        tb = floor_t2(tb);
       }
       const float2 xa = ex2x2(ta), xb = ex2x2(tb);
       s0 = fadd2(s0, xa);
@@ -123,10 +121,7 @@ __device__ __forceinline__ void sum_pass(const uint4* sv, int n_vec, float k, fl
 #pragma unroll
     for (int e = 0; e < P; ++e) {
       float2 ta = ffma2(fa[e], k2, nm2);
-      if (kSafe) {
-        if (fa[e].x == -INFINITY) ta.x = -127.0f;
-        if (fa[e].y == -INFINITY) ta.y = -127.0f;
-      }
+      if (kSafe) ta = floor_t2(ta);
       const float2 xa = ex2x2(ta);
       s0 = fadd2(s0, xa);
       u0 = ffma2(xa, ta, u0);
@@ -137,16 +132,16 @@ __device__ __forceinline__ void sum_pass(const uint4* sv, int n_vec, float k, fl
   u_out = u.x + u.y;
 }
 
-// The thread's sums against its own maximum over the slice, skipping -inf
-// logits exactly: the rare path (no finite first vector, an overflow, or a
-// -inf logit).
+// The thread's sums against its own maximum over the slice, skipping masked
+// logits exactly: the rare path (no logit in the first vector, an overflow, or
+// a masked logit).
 template <class In, int kThreads>
 __device__ __forceinline__ Tri slow_sums(const uint4* sv, int n_vec, float k) {
   typename In::MaxAcc macc = In::kMaxInit;
   for (int v = threadIdx.x; v < n_vec; v += kThreads) macc = In::max_acc(macc, sv[v]);
   const float r = In::max_val(macc) * k;
   Tri t{-INFINITY, 0.0f, 0.0f};
-  if (r != -INFINITY) {
+  if (!(r < kNoLogit)) {
     float su, uu;
     sum_pass<In, kThreads, true>(sv, n_vec, k, r, su, uu);
     t = Tri{r, su, uu};
@@ -295,9 +290,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep(const SweepArgs 
 
     // ---------------- pass A: one sweep against the maximum of the thread's
     // first vector. The sums stay finite unless a logit lies more than
-    // 127 / k above that reference; that case (inf) or a -inf logit (NaN)
+    // 127 / k above that reference; that case (inf) or a masked logit (NaN)
     // takes the thread's maximum over the slice and sums again, skipping
-    // -inf logits exactly. Sums past 2^16 move the reference up by their
+    // masked logits exactly. Sums past 2^16 move the reference up by their
     // binary exponent (an exact rescale) before the merge.
     Tri t{-INFINITY, 0.0f, 0.0f};
     if (have && tid < n_vec) {
@@ -318,8 +313,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_sweep(const SweepArgs 
     }
     for (int j = vec_elems + tid; j < cnt; j += kThreads) {  // elements past the vectors
       const float z = In::load1(grow, j);
-      if (z == -INFINITY) continue;
       const float zk = z * k;
+      if (zk < kNoLogit) continue;
       if (zk > t.m) {
         if (t.s > 0.0f) {
           const float d = t.m - zk, f = ex2(d);

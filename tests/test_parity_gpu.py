@@ -673,6 +673,35 @@ def test_topk_candidate_of_probability_zero(name, vocab, mode):
         P.assert_dlogits_close(g["dlogits_t"].float().cpu().numpy(), o["dlogits"])
 
 
+@pytest.mark.parametrize("name,vocab", [
+    ("glm", 2048), ("glm", 9600), ("glm", 12288), ("glm", 45056), ("glm", 65792), ("glm", 151936),
+    ("glm", 262144), ("glm", 701), ("glm", 45003), ("fp32", 1024), ("fp32", 32768), ("fp32", 10001)])
+@pytest.mark.parametrize("temperature", [1.0, 2.0])
+def test_masked_with_the_lowest_finite_value(name, vocab, temperature):
+    """Logits of the type's lowest value, as masks leave them, have probability
+    zero like -inf: scaled they overflow to it (T = 1), or not (T = 2), then
+    with a rounding error far above 1. Single ones, whole vectors, and a third
+    of the row, which leaves some threads nothing else."""
+    rec = wl.shrink(wl.RECIPES[name], n_prompts=1, group_size=2, traj_len=3, vocab=vocab,
+                    rho_noise=0.3, mask="none")
+    w = wl.make(rec, DEV)
+    low = torch.finfo(w.logits.dtype).min
+    w.targets.fill_(vocab - 1)
+    w.logits[1, 5] = w.logits[1, vocab - 2] = low
+    w.logits[2, :vocab // 3] = low
+    w.logits[3, vocab // 4:vocab - 1] = low
+    w.logits[4, ::2] = low
+    w.logits[4, vocab - 1] = 2.0
+    w.logits[5, 16:32] = -float("inf")
+    w.logits[5, 64:400] = low
+    params = dict(w.params, temperature=temperature, entropy_coef=0.01)
+    w.rollout_logprobs.copy_(torch.from_numpy(P.run_oracle(w, params=params)["logp"]).float() + 0.1)
+    if w.ref_logprobs is not None:
+        w.ref_logprobs.copy_(w.rollout_logprobs)
+    _full_check(w, params=params)
+    _full_check(w, mode="split", params=params)
+
+
 @pytest.mark.parametrize("kind,cluster", [("cluster", 0), ("cluster", 4), ("stream", 0)])
 def test_topk_ids_out_of_range_are_reported(ov, kind, cluster):
     """A top-K OPD candidate id outside [0, vocab) zeros its row (as a bad
