@@ -538,10 +538,6 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
   const size_t traj_bytes = (4 * static_cast<size_t>(f.n_traj) + 1) * sizeof(int);
   aa.smem_traj = traj_bytes <= static_cast<size_t>(kAdvSmemBytes);
   aa.ws = ws;
-  // Small calls, where launches count, start while whatever ran before them
-  // ends (eager calls of 2,048 x 4,096 23.1 -> 20 us); past that the waiting
-  // CTAs are in the way as often as they help (3,488 x 43,648 with top-K 127.0
-  // -> 132.0 us, two vocabulary shards of 4,096 rows 657 -> 645).
   bool grpo = aa.estimator == RL_EST_GRPO && aa.smem_traj && aa.n_traj > 0 && !aa.counts_out;
   aa.groups_done = group_kernel_pays(grpo, f.n_groups, f.n_traj);
   if (aa.groups_done) grpo = false;

@@ -11,12 +11,22 @@ namespace milesloss {
 constexpr int kMaxStages = 4;
 constexpr int kMaxCluster = 8;
 constexpr uint32_t kBulkChunk = 16384;    // bytes per cp.async.bulk
-constexpr int kEarlyStartRows = 2048;     // calls of up to this many rows overlap what ran before
+// Calls of up to this many rows start while what ran before them ends (their
+// first kernel waits there for it). That gives about a launch, 1 to 3 us, at any
+// size, so the line is where it is some per cent of a call. Late / early, us,
+// calls back to back: 1,024 x 8,192 bf16 16.4 / 15.0, 2,048 x 4,096 16.7 / 15.4,
+// 4,096 x 4,096 26.1 / 26.6, 8,192 x 4,096 38.1 / 38.4; streamed, 2,048 x 32,768 56.3 /
+// 54.7, 8,192 x 32,768 182.7 / 180.8, 4,096 x 151,936 408.5 / 407.7. The cluster
+// kernel loses by it back to back and gains behind another kernel (a matrix
+// product of 14 us included): 2,048 x 45,056 75.5 / 78.2 and 90.8 / 86.3, 8,192 x
+// 45,056 247.8 / 255.2 and 265.7 / 260.9, with top-K 2,048 x 43,648 81.0 / 84.2 and
+// 95.3 / 92.6.
+constexpr int kEarlyStartRows = 2048;
 constexpr int kAdvThreads = 512;
-// CTAs of the advantage kernel (one cluster). With 1 / 4 / 8: 512 trajectories of
-// 64 rows x 32,768 fp32 1,426 / 1,337 / 1,327 us a call, 128 x 128 rows x 20,480
-// (forward) 144 / 131 / 127, 16,384 rows x 151,936 1,548 / 1,535 / 1,533; the same to
-// 1 us on 2,048 rows x 4,096.
+// CTAs of k_advantages (one cluster). With 1 / 4 / 8, us a call: REINFORCE++, 128
+// trajectories of 4 rows x 2,048 39.4 / 26.1 / 24.2, 512 of 4 141 / 54 / 40, 4,096 of 4
+// 804 / 274 / 186, 128 of 64 rows x 20,480 154 / 140 / 138; GSPO, 2,048 of 4 306 / 141 /
+// 117; 16 trajectories 22.9 / 22.2 / 21.9.
 constexpr int kAdvCluster = 8;
 constexpr int kBwdThreads = 256;
 // k_stream's block: cw consumer warps (16 with one CTA per SM, 8 with two, 4
