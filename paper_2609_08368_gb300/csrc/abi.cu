@@ -788,12 +788,16 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     pdl = overlap;
   }
 
-  // GSPO's gradient, from the trajectories' terms. After a sweep that fills the
-  // shared memory it is no dependent: its blocks would start on SMs still set
-  // up for that, with 28 KB of L1 for their loads in flight (8,192 x 151,936
-  // bf16: 1,225 us that way, 1,080 before any kernel overlapped).
-  if (gspo && go && (phase & RL_PHASE_ROWS) && call.R > 0) {
-    st = launch_bwd(call, *go, ws_all, s, 0, pdl && small_smem);
+  // GSPO's gradient, from the trajectories' terms. After k_short it comes before
+  // the statistics, as a dependent (4,096 x 4,096 68 us with neither, 45 now).
+  // After a sweep that fills the shared memory it is no dependent: its blocks
+  // would start on SMs still set up for that, with 28 KB of L1 for their loads in
+  // flight (8,192 x 151,936 bf16: 1,225 us that way, 1,061 not); and it comes last
+  // (65,536 x 154,880: 8,110 us, before the statistics 8,160; 8,192 x 151,936 1,060
+  // and 1,061).
+  const bool grad_pass = gspo && go && (phase & RL_PHASE_ROWS) && call.R > 0;
+  if (grad_pass && small_smem) {
+    st = launch_bwd(call, *go, ws_all, s, 0, pdl);
     if (st != RL_OK) return st;
     pdl = overlap;
   }
@@ -803,6 +807,7 @@ rl_status run_fwd(const FwdIn& f, const GradOut* go, cudaStream_t s, int phase =
     if (st != RL_OK) return st;
     pdl = overlap;
   }
+  if (grad_pass && !small_smem) return launch_bwd(call, *go, ws_all, s, 0, false);
   return RL_OK;
 }
 

@@ -86,3 +86,17 @@ def test_short_rows_with_topk_take_the_faster_kernel(dtype, vocab, topk, mode):
     with ml.launch_overrides(sweep_kernel="cluster"):
         other = _fastest(call)
     assert chosen <= 1.06 * other, (chosen, other)
+
+
+def test_gradient_sweep_of_fp32_rows_runs_at_the_copy_rate():
+    """Of 32,768 rows x 32,768: its bytes (the training rows' logits, every
+    dLogit) in little more than the time a copy of as many takes."""
+    w = wl.make(wl.shrink(wl.RECIPES["fp32"], n_prompts=64, group_size=8, traj_len=64), DEV)
+    buf = api.alloc(w.n_rows, 512, w.n_groups, DEV, vocab=w.vocab, dlogits_dtype=w.logits.dtype)
+    api.fwd(w, buf)
+    sweep = _fastest(lambda: api.bwd(w, buf), reps=8)
+    trains = float((w.loss_mask != 0).float().mean())
+    half = int(w.logits.numel() * (1 + trains) / 2)  # elements read, and as many written
+    src, dst = w.logits.view(-1)[:half], buf.dlogits.view(-1)[:half]
+    copy = _fastest(lambda: dst.copy_(src), reps=8)
+    assert sweep <= 1.04 * copy, (sweep, copy)
