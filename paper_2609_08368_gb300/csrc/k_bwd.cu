@@ -61,9 +61,12 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd(const BwdArgs a) {
   // rows that do not train (or have a bad target) get zeros: no read
   auto reads = [&](long long row) { return a.mask[row] != 0 && !(ws.flags[row] & kFlagBad); };
   // (rd: whether the row is read; the block's first tile is loaded before the
-  // kernel in front has finished, so by the mask alone. fp32 asks for the
-  // others in here: asked by the caller it took 1,158 us instead of 1,112 on 32,768 x
-  // 32,768, where bf16, asked in here, loses 0.3 % of a GSPO call.)
+  // kernel in front has finished, so by the mask alone. bf16 asks for the next
+  // tile once and carries the answer over, fp32 asks in here and again: us, bf16
+  // 131,072 x 151,936 (T = 0.7) carried 8,560, asked twice 8,760, in here 8,670,
+  // 65,536 x 154,880 5,365 / 5,415 / 5,490; fp32 32,768 x 32,768 1,143 / 1,158 /
+  // 1,115. Known two tiles ahead it is 7,190 on the first and 1-4 % slower on
+  // other calls.)
   constexpr bool kAskInside = V8 == 4;
   auto load_tile = [&](long long row, int t, uint4* raw, bool rd, bool first) {
     const char* zrow;
@@ -88,11 +91,13 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd(const BwdArgs a) {
   float g = a.grad_loss;
   if (a.grad_loss_dev) g *= *a.grad_loss_dev;
   const float cscale = (N > 0) ? g / static_cast<float>(N) * a.invT : 0.0f;
+  bool rd = !kAskInside && row < a.R && reads(row);
   while (row < a.R) {
     long long nrow = row;
     int nt = t;
     advance(nrow, nt);
-    if (nrow < a.R) load_tile(nrow, nt, nxt, kAskInside || reads(nrow), false);
+    const bool rd_next = !kAskInside && nrow < a.R && reads(nrow);
+    if (nrow < a.R) load_tile(nrow, nt, nxt, rd_next, false);
     const char* zrow;
     char* drow;
     row_ptrs(row, zrow, drow);
@@ -102,7 +107,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd(const BwdArgs a) {
     const int jv = t * kTile + (kUnal ? max(head, 0) : 0);
     const int j0 = (kUnal && t == 0) ? 0 : min(a.V, jv);
     const int j1 = (kUnal && t == tpr - 1) ? a.V : min(a.V, jv + kTile);
-    const bool rd = reads(row);
+    if (kAskInside) rd = reads(row);
     const float cc = rd ? cscale : 0.0f;
     const float G = ws.G[row], H = ws.H[row], lse = ws.lse[row];
     const float ca = cc * (-G + a.gamma * (H - lse));
@@ -167,6 +172,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd(const BwdArgs a) {
     for (int i = 0; i < kPer; ++i) raw[i] = nxt[i];
     row = nrow;
     t = nt;
+    rd = rd_next;
   }
 }
 
